@@ -164,8 +164,8 @@ struct Launch {
   int32_t total_units = 0;
   int32_t max_n = 0;
   int64_t cells = 0;     // sum of N * M over the launch (tuning bucket)
-  int grid_x = 1;
   double bytes = 0, flops = 0;
+  FinLaunch fin, fin_gram; // FIN launches
   GramPlan gp;             // GRAM launches
   int iso_mode = 0;
   // E4M3 member scales to compute before the Gram launch: by a pass of their own, or from
@@ -351,8 +351,8 @@ static pid_status plan_batch(pid_handle h, const pid_ensemble* ens, int count, c
   const size_t fdesc_bytes = align_up(static_cast<int64_t>(n_f) * sizeof(FinDesc), 256);
   bp->desc_bytes = sdesc_bytes + fdesc_bytes;
   size_t off = bp->desc_bytes;
-  std::vector<double*> part(count), sums(count);
-  std::vector<float*> coef(count), gpart(count, nullptr);
+  std::vector<double*> sums(count);
+  std::vector<float*> part(count), coef(count), gpart(count, nullptr);
   std::vector<float*> scale(count, nullptr);
   // Operand planes of the tiled Gram: written by the streaming pass into one buffer per
   // ensemble (BF16, store_u), else staged into one buffer reused by the launches in turn.
@@ -380,7 +380,7 @@ static pid_status plan_batch(pid_handle h, const pid_ensemble* ens, int count, c
     const int o = owner(e);
     if (o == e) {
       const size_t pb = is_gram[e] && !tiled[e] ? std::max(pl[e].part_bytes, gp[e].part_bytes) : pl[e].part_bytes;
-      part[e] = reinterpret_cast<double*>(base + off); off += pb * steps;
+      part[e] = reinterpret_cast<float*>(base + off); off += pb * steps;
       sums[e] = reinterpret_cast<double*>(base + off); off += pl[e].sums_bytes;
       coef[e] = reinterpret_cast<float*>(base + off); off += pl[e].coef_bytes;
       if (is_gram[e]) {
@@ -472,7 +472,6 @@ static pid_status plan_batch(pid_handle h, const pid_ensemble* ens, int count, c
     f.kind = kind;
     f.sums = sums[e];
     f.coef = coef[e];
-    f.ticket = h->tickets + e;
     const pid_ensemble& o = ens[e];
     if (kind != FIN_LIN1) {
       f.depth = o.depth; f.in_in = o.in_in; f.in_out = o.in_out; f.rank = o.rank;
@@ -485,6 +484,7 @@ static pid_status plan_batch(pid_handle h, const pid_ensemble* ens, int count, c
     if (kind == FIN_GRAM) {
       f.gpart = gpart[e];
       f.n_gchunks = steps * gram_chunks(e);
+      f.gram_inline = fin_gram_inline(f.N, f.n_gchunks) ? 1 : 0;
       f.P = o.P;
       f.err_est = o.err_est;
       if (sib[e] >= 0) {   // (m, A) from the first streaming pass over the same masks
@@ -492,9 +492,23 @@ static pid_status plan_batch(pid_handle h, const pid_ensemble* ens, int count, c
         f.n_chunks = pl[sib[e]].desc.n_chunks;
       }
     }
-    const int nb = (2 * f.N + 31) / 32 + (kind == FIN_GRAM ? fin_gram_items(f.N) : 0);
-    f.slices = std::max(1, std::min(nb, 2 * h->sms));
     return f;
+  };
+  // The finalisation of one phase over the ensembles `which` selects: the Gram ensembles'
+  // descriptors follow the others'.
+  auto add_fin = [&](auto&& which, auto&& kind_of) {
+    Launch L;
+    L.kind = Launch::FIN;
+    L.first = static_cast<int>(bp->fdesc.size());
+    for (const bool gram : {false, true}) {
+      for (int e = 0; e < count; ++e) {
+        if (owner(e) != e || !which(e) || (kind_of(e) == FIN_GRAM) != gram) continue;
+        bp->fdesc.push_back(fin_for(e, kind_of(e)));
+        fin_launch_add(gram ? &L.fin_gram : &L.fin, bp->fdesc.back());
+      }
+    }
+    L.count = static_cast<int>(bp->fdesc.size()) - L.first;
+    bp->launches.push_back(L);
   };
 
   // Phase 1: first streaming passes (which may also reduce E4M3 maxima), then the Gram
@@ -546,32 +560,12 @@ static pid_status plan_batch(pid_handle h, const pid_ensemble* ens, int count, c
     L.scale_from_keys = keys_src[e] >= 0;
     bp->launches.push_back(L);
   }
-  {
-    Launch L;
-    L.kind = Launch::FIN;
-    L.first = static_cast<int>(bp->fdesc.size());
-    for (int e = 0; e < count; ++e) {
-      if (owner(e) != e) continue;
-      const int kind = is_gram[e] ? FIN_GRAM : (is_lin[e] ? FIN_LIN1 : FIN_MEAN);
-      bp->fdesc.push_back(fin_for(e, kind));
-      L.grid_x = std::max(L.grid_x, bp->fdesc.back().slices);
-    }
-    L.count = static_cast<int>(bp->fdesc.size()) - L.first;
-    bp->launches.push_back(L);
-  }
+  add_fin([&](int) { return true; },
+          [&](int e) { return is_gram[e] ? FIN_GRAM : (is_lin[e] ? FIN_LIN1 : FIN_MEAN); });
   // Phase 2: exact full PID, second streaming pass and its finalisation.
   if (n_lin) {
     for (auto& kv : pass2) add_stream_class(kv.second, true);
-    Launch L;
-    L.kind = Launch::FIN;
-    L.first = static_cast<int>(bp->fdesc.size());
-    for (int e = 0; e < count; ++e) {
-      if (!is_lin[e] || owner(e) != e) continue;
-      bp->fdesc.push_back(fin_for(e, FIN_LIN2));
-      L.grid_x = std::max(L.grid_x, bp->fdesc.back().slices);
-    }
-    L.count = static_cast<int>(bp->fdesc.size()) - L.first;
-    bp->launches.push_back(L);
+    add_fin([&](int e) { return is_lin[e] != 0; }, [&](int) { return FIN_LIN2; });
   }
   return PID_OK;
 }
@@ -587,7 +581,7 @@ static pid_status enqueue(pid_handle h, const BatchPlan& bp, char* base, const v
   const EnsDesc* sdev = reinterpret_cast<const EnsDesc*>(base);
   const size_t sdesc_bytes = align_up(static_cast<int64_t>(bp.sdesc.size()) * sizeof(EnsDesc), 256);
   const FinDesc* fdev = reinterpret_cast<const FinDesc*>(base + sdesc_bytes);
-  auto launch_one = [&](const Launch& L, cudaStream_t s) -> pid_status {
+  auto launch_one = [&](const Launch& L, cudaStream_t s, bool follows) -> pid_status {
     cudaError_t e = cudaSuccess;
     if (L.kind == Launch::STREAM) {
       StreamParams sp;
@@ -632,7 +626,26 @@ static pid_status enqueue(pid_handle h, const BatchPlan& bp, char* base, const v
       fp.n_ens = L.count;
       fp.err = h->err_word;
       ProfScope ps(h, PID_KERNEL_FINALIZE, 0.0, 0.0, s);
-      e = launch_finalize(fp, L.grid_x, L.count, s);
+      // the Gram ensembles' launches run beside the others' on a side stream
+      BatchCache* c = h->batch;
+      const bool both = L.fin.count > 0 && L.fin_gram.count > 0;
+      const bool fork = both && c && c->fork_ev;
+      FinParams fg = fp;
+      fg.descs = fp.descs + L.fin.count;
+      FinLaunch l0 = L.fin, l1 = L.fin_gram;
+      l0.pdl = follows && !both;
+      l1.pdl = follows && !both;
+      const cudaStream_t sg = fork ? c->side[0] : s;
+      if (fork) {
+        e = cudaEventRecord(c->fork_ev, s);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(sg, c->fork_ev, 0);
+      }
+      if (e == cudaSuccess && l1.count) e = launch_finalize(fg, l1, sg);
+      if (e == cudaSuccess && l0.count) e = launch_finalize(fp, l0, s);
+      if (e == cudaSuccess && fork) {
+        e = cudaEventRecord(c->join_ev[0], sg);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(s, c->join_ev[0], 0);
+      }
       if (e != cudaSuccess) return cuda_fail(h, e, "batch finalize launch");
     }
     return PID_OK;
@@ -643,6 +656,7 @@ static pid_status enqueue(pid_handle h, const BatchPlan& bp, char* base, const v
   // GPU on their own and run in order on `s`.
   BatchCache* c = h->batch;
   const size_t n = bp.launches.size();
+  bool on_s = false;   // the last thing enqueued on `s` is a kernel
   for (size_t i = 0; i < n;) {
     const Launch::Kind kind = bp.launches[i].kind;
     size_t j = i + 1;
@@ -650,17 +664,20 @@ static pid_status enqueue(pid_handle h, const BatchPlan& bp, char* base, const v
       while (j < n && bp.launches[j].kind == kind) ++j;
     if (j - i == 1 || !c || !c->fork_ev) {
       for (size_t k = i; k < j; ++k) {
-        const pid_status st = launch_one(bp.launches[k], s);
+        // a finalisation right behind a kernel on `s` may be launched while it still runs
+        const pid_status st = launch_one(bp.launches[k], s, k > 0 && on_s);
         if (st != PID_OK) return st;
+        on_s = true;
       }
     } else {
+      on_s = false;
       if ((e = cudaEventRecord(c->fork_ev, s)) != cudaSuccess) return cuda_fail(h, e, "fork");
       const int used = static_cast<int>(std::min<size_t>(j - i, BatchCache::kSide));
       for (int k = 0; k < used; ++k)
         if ((e = cudaStreamWaitEvent(c->side[k], c->fork_ev, 0)) != cudaSuccess)
           return cuda_fail(h, e, "fork");
       for (size_t k = i; k < j; ++k) {
-        const pid_status st = launch_one(bp.launches[k], c->side[(k - i) % BatchCache::kSide]);
+        const pid_status st = launch_one(bp.launches[k], c->side[(k - i) % BatchCache::kSide], false);
         if (st != PID_OK) return st;
       }
       for (int k = 0; k < used; ++k) {

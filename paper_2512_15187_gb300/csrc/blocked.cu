@@ -12,7 +12,7 @@
 // With c_j = 1 this is PID-mean's pass (A_i = N x the sum against u_bar, Eq. 15-16); with
 // c_j = 1/(N m_j) it is the second pass of the exact full PID (IN_out of Eq. 10 with the
 // sums of Eq. 14). The isovalue map of Sec. 3.5 is applied to each element as it is read.
-// rank_kernel ranks more members than the finalisation's single CTA holds.
+// rank_kernel ranks the members.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -34,7 +34,7 @@ struct BlockedParams {
   const float* coef;     // [N] column-sum coefficients, or nullptr (every c_j = 1)
   float* S;              // [n_blocks][ldS] per-block column sums
   float* s;              // [ldS] combined column sum
-  double* part;          // [n_chunks][2N]
+  float* part;           // [n_chunks][2N]
   int64_t N, M, ld, ldS;
   int32_t n_blocks, n_chunks;
   int32_t iso_mode;
@@ -132,8 +132,8 @@ __global__ void __launch_bounds__(256) accum_kernel(const __grid_constant__ Bloc
   m = warp_sum(m);
   a = warp_sum(a);
   if (lane == 0) {
-    p.part[c * 2 * p.N + i] = static_cast<double>(m);
-    p.part[c * 2 * p.N + p.N + i] = static_cast<double>(a);
+    p.part[c * 2 * p.N + i] = m;
+    p.part[c * 2 * p.N + p.N + i] = a;
   }
 }
 
@@ -194,13 +194,12 @@ pid_status run_blocked(pid_handle h, const EnsInput& in, const EnsOutputs& out, 
   const int64_t ldS = rup(M, 4);
   const int n_blocks = static_cast<int>((N + kBlockRows - 1) / kBlockRows);
   const int n_chunks = static_cast<int>((M + kAccChunk - 1) / kAccChunk);
-  const bool big = N > 1024;                      // ranks beyond the finalisation's CTA
   const size_t S_bytes = rup(static_cast<int64_t>(n_blocks) * ldS * 4, 256);
   const size_t s_bytes = rup(ldS * 4, 256);
-  const size_t part_bytes = rup(static_cast<int64_t>(n_chunks) * 2 * N * 8, 256);
+  const size_t part_bytes = rup(static_cast<int64_t>(n_chunks) * 2 * N * 4, 256);
   const size_t sums_bytes = rup(4 * N * 8, 256);
   const size_t coef_bytes = rup(N * 4, 256);
-  const size_t dtmp_bytes = (big && out.rank && !out.depth) ? rup(N * 8, 256) : 0;
+  const size_t dtmp_bytes = (out.rank && !out.depth) ? rup(N * 8, 256) : 0;
   pid_status st = ensure_workspace(h, S_bytes + s_bytes + part_bytes + sums_bytes + coef_bytes +
                                           dtmp_bytes, s);
   if (st != PID_OK) return st;
@@ -209,7 +208,7 @@ pid_status run_blocked(pid_handle h, const EnsInput& in, const EnsOutputs& out, 
   std::memset(&p, 0, sizeof(p));
   p.S = reinterpret_cast<float*>(ws);
   p.s = reinterpret_cast<float*>(ws + S_bytes);
-  p.part = reinterpret_cast<double*>(ws + S_bytes + s_bytes);
+  p.part = reinterpret_cast<float*>(ws + S_bytes + s_bytes);
   double* sums = reinterpret_cast<double*>(ws + S_bytes + s_bytes + part_bytes);
   float* coef = reinterpret_cast<float*>(ws + S_bytes + s_bytes + part_bytes + sums_bytes);
   double* dtmp = dtmp_bytes ? reinterpret_cast<double*>(ws + S_bytes + s_bytes + part_bytes +
@@ -231,7 +230,6 @@ pid_status run_blocked(pid_handle h, const EnsInput& in, const EnsOutputs& out, 
   fd.depth = out.depth ? out.depth : dtmp;
   fd.in_in = out.in_in;
   fd.in_out = out.in_out;
-  fd.rank = big ? nullptr : out.rank;
   fd.mass = out.mass;
   fd.mean_depth = out.mean_depth;
 
@@ -258,7 +256,7 @@ pid_status run_blocked(pid_handle h, const EnsInput& in, const EnsOutputs& out, 
     f2.mass = nullptr; f2.mean_depth = nullptr;
     if ((st = launch_fin_one(h, f2, s)) != PID_OK) return st;
   }
-  if (big && out.rank) {
+  if (out.rank) {
     const unsigned slices = static_cast<unsigned>(N / 4096 < 1 ? 1 : (N / 4096 > 16 ? 16 : N / 4096));
     cudaError_t e = cudaMemsetAsync(out.rank, 0, static_cast<size_t>(N) * sizeof(int32_t), s);
     if (e != cudaSuccess) return cuda_fail(h, e, "rank reset");

@@ -407,7 +407,7 @@ pid_status plan_stream(pid_handle h, const EnsInput& in, EnsPlan* pl) {
   const int64_t stage_rows = pl->cls ? int64_t(d.n_cls) * d.n_boxes * d.box_rows
                                      : int64_t(d.n_boxes) * d.box_rows;
   pl->stage_floats = static_cast<int32_t>(round_up(stage_rows * row_floats + TS, 32));
-  pl->part_bytes = round_up(static_cast<int64_t>(d.n_chunks) * 2 * in.N * 8, 256);
+  pl->part_bytes = round_up(static_cast<int64_t>(d.n_chunks) * 2 * in.N * 4, 256);
   pl->sums_bytes = round_up((4 * in.N + in.N * in.N) * 8, 256);
   pl->coef_bytes = round_up(in.N * 4, 256);
   return PID_OK;
@@ -584,17 +584,19 @@ static pid_status launch_stream_one(pid_handle h, EnsPlan& pl, const float* coef
 }
 
 pid_status launch_fin_one(pid_handle h, FinDesc fd, cudaStream_t s) {
-  const int nb_stream = (2 * fd.N + 31) / 32;
-  const int nb_gram = fd.kind == FIN_GRAM ? fin_gram_items(fd.N) : 0;
-  fd.slices = std::max(1, std::min(nb_stream + nb_gram, 2 * h->sms));
   FinParams fp;
   std::memset(&fp, 0, sizeof(fp));
+  const bool large = fd.N > kMaxMembers;
+  if (large) fd.slices = std::max(1, std::min((2 * fd.N + 31) / 32, 2 * h->sms));
+  FinLaunch l;
+  fin_launch_add(&l, fd);
+  l.pdl = true;   // the kernel before it in the stream wrote its partials
   fp.one = fd;
   fp.descs = nullptr;
   fp.n_ens = 1;
   fp.err = h->err_word;
   ProfScope ps(h, PID_KERNEL_FINALIZE, 0.0, 0.0, s);
-  cudaError_t e = launch_finalize(fp, fd.slices, 1, s);
+  cudaError_t e = large ? launch_finalize_large(fp, s) : launch_finalize(fp, l, s);
   if (e != cudaSuccess) return cuda_fail(h, e, "finalize launch");
   return PID_OK;
 }
@@ -623,7 +625,7 @@ static pid_status run_gram_tiled(pid_handle h, const EnsInput& in, EnsPlan& pl,
   st = ensure_workspace(h, off_op + tp.op_bytes, s);
   if (st != PID_OK) return st;
   char* ws = static_cast<char*>(h->ws);
-  double* part = reinterpret_cast<double*>(ws);
+  float* part = reinterpret_cast<float*>(ws);
   float* gpart = reinterpret_cast<float*>(ws + off_gpart);
   pl.desc.part = part;
   // BF16 operands come straight from the streaming pass (its one-cell-per-lane classes,
@@ -653,9 +655,9 @@ static pid_status run_gram_tiled(pid_handle h, const EnsInput& in, EnsPlan& pl,
   fd.n_chunks = pl.desc.n_chunks;
   fd.gpart = gpart;
   fd.n_gchunks = tp.n_gchunks;
+  fd.gram_inline = fin_gram_inline(fd.N, fd.n_gchunks) ? 1 : 0;
   fd.sums = reinterpret_cast<double*>(ws + off_sums);
   fd.coef = reinterpret_cast<float*>(ws + off_coef);
-  fd.ticket = h->tickets;
   fd.depth = out.depth;
   fd.in_in = out.in_in;
   fd.in_out = out.in_out;
@@ -686,7 +688,7 @@ pid_status run_single(pid_handle h, const EnsInput& in, const EnsOutputs& out, c
   st = ensure_workspace(h, need, s);
   if (st != PID_OK) return st;
   char* ws = static_cast<char*>(h->ws);
-  double* part = reinterpret_cast<double*>(ws);
+  float* part = reinterpret_cast<float*>(ws);
   double* sums = reinterpret_cast<double*>(ws + part_bytes);
   float* coef = reinterpret_cast<float*>(ws + part_bytes + pl.sums_bytes);
   char* gbase = ws + part_bytes + pl.sums_bytes + pl.coef_bytes;
@@ -699,7 +701,6 @@ pid_status run_single(pid_handle h, const EnsInput& in, const EnsOutputs& out, c
   fd.n_chunks = pl.desc.n_chunks;
   fd.sums = sums;
   fd.coef = coef;
-  fd.ticket = h->tickets;
   fd.depth = out.depth;
   fd.in_in = out.in_in;
   fd.in_out = out.in_out;
@@ -728,6 +729,7 @@ pid_status run_single(pid_handle h, const EnsInput& in, const EnsOutputs& out, c
     fd.n_chunks = own_pass ? pl.desc.n_chunks : gp.n_gchunks;
     fd.gpart = gpart;
     fd.n_gchunks = gp.n_gchunks;
+    fd.gram_inline = fin_gram_inline(fd.N, fd.n_gchunks) ? 1 : 0;
     fd.P = out.P;
     fd.err_est = out.err_est;
     return launch_fin_one(h, fd, s);
@@ -955,7 +957,7 @@ pid_status pid_autotune_shapes(pid_handle h, const pid_ensemble* ens, int32_t co
         EnsPlan pl;
         if ((st = plan_stream(h, in, &pl)) != PID_OK) break;
         if ((st = ensure_workspace(h, pl.part_bytes, s)) != PID_OK) break;
-        pl.desc.part = static_cast<double*>(h->ws);
+        pl.desc.part = static_cast<float*>(h->ws);
         const float ms = time_runs(s, 3, [&] { return launch_stream_one(h, pl, nullptr, s); }, &st);
         if (st != PID_OK) break;
         if (ms < best) { best = ms; pick = c; }
@@ -977,7 +979,7 @@ pid_status pid_autotune_shapes(pid_handle h, const pid_ensemble* ens, int32_t co
           const size_t need = gp.part_bytes + kScaleBytes + gp.gpart_bytes;
           if ((st = ensure_workspace(h, need, s)) != PID_OK) break;
           char* ws = static_cast<char*>(h->ws);
-          double* part = reinterpret_cast<double*>(ws);
+          float* part = reinterpret_cast<float*>(ws);
           float* scale = reinterpret_cast<float*>(ws + gp.part_bytes);
           float* gpart = reinterpret_cast<float*>(ws + gp.part_bytes + kScaleBytes);
           const float ms =

@@ -16,7 +16,7 @@ namespace pidh {
 
 constexpr int64_t kMaxMembers = 512;   // largest N of the fused single-pass kernels
 constexpr int64_t kMaxBlockedMembers = int64_t(1) << 22;   // single calls, member-blocked path
-constexpr int kMaxTickets = 8192;      // ensembles per batch (one finalisation ticket each)
+constexpr int kMaxTickets = 8192;      // ensembles per batch
 constexpr int64_t kMaxMatrixMembers = 65536;   // members of pid_depth_from_matrix
 constexpr int kMaxSpacetimeSteps = 65536;   // time steps of one space-time ensemble
 
@@ -132,7 +132,7 @@ struct GramPlan {
   size_t smem = 0;
   bool exact = true;       // false: soft masks whose (m, A) come from a streaming pass
   size_t gpart_bytes = 0;  // [n_gchunks][N][N] float32
-  size_t part_bytes = 0;   // [n_gchunks][2N] float64 (exact PID-mean partials)
+  size_t part_bytes = 0;   // [n_gchunks][2N] float32 (exact PID-mean partials)
   double bytes = 0, flops = 0;
 };
 
@@ -177,6 +177,14 @@ pid_status check_shape(pid_handle h, const void* data, int64_t N, int64_t M, int
 pid_status launch_member_coef_one(pid_handle h, const double* r, int64_t N, float* coef,
                                   cudaStream_t s);
 pid_status launch_fin_one(pid_handle h, pidk::FinDesc fd, cudaStream_t s);
+// Counts one ensemble into a finalisation launch.
+inline void fin_launch_add(pidk::FinLaunch* l, const pidk::FinDesc& fd) {
+  ++l->count;
+  l->max_n = fd.N > l->max_n ? fd.N : l->max_n;
+  l->gram = l->gram || fd.kind == pidk::FIN_GRAM;
+  l->sum_gram = l->sum_gram || (fd.kind == pidk::FIN_GRAM && !fd.gram_inline);
+  l->matrix = l->matrix || (fd.P != nullptr && fd.N > pidk::kFinInlineMatrixN);
+}
 pid_status run_blocked(pid_handle h, const EnsInput& in, const EnsOutputs& out, cudaStream_t s);
 pid_status check_opt(pid_handle h, const pid_options* o);
 pid_status plan_stream(pid_handle h, const EnsInput& in, EnsPlan* pl);
@@ -224,7 +232,7 @@ pid_status launch_scales_from_keys(pid_handle h, int64_t N, float* region, cudaS
 pid_status plan_gram(pid_handle h, const EnsInput& in, GramPlan* gp);
 void gram_geometry(pid_handle h, int G, int mpw, bool wide, int prec, int32_t stage_floats,
                    int* dF, int* dO, size_t* smem);
-pid_status launch_gram_one(pid_handle h, const EnsInput& in, GramPlan& gp, double* part,
+pid_status launch_gram_one(pid_handle h, const EnsInput& in, GramPlan& gp, float* part,
                            float* gpart, float* scale, cudaStream_t s, bool scales_ready = false);
 // Gram launch over `count` device descriptors (part / gpart / op_scale already set).
 pid_status launch_gram_batch(pid_handle h, const GramPlan& gp, const pidk::EnsDesc* descs,

@@ -1,0 +1,673 @@
+// Finalisation: fixed-order reduction of the per-chunk partials, then the inclusion
+// fractions, depths and ranks of Eq. 10 / Eq. 16, and the calibration of the tensor-core
+// Gram.
+//
+// One cluster of kFinCtas CTAs per ensemble of up to 512 members; CTA r owns a contiguous
+// block of members from the partials to their ranks. What one member needs from all the
+// others (the mean contour's mass, the calibration scales, the order keys of the depths) is
+// pushed into every CTA's shared memory and separated by cluster barriers, so a finalisation
+// is one launch without tickets or round trips through L2.
+//
+// What bounds it is latency: a chain of an L2 read, a few FP64 operations and barriers. GB300
+// issues two FP64 operations per clock and SM, so
+//   * the partials, which are FP32 values, are summed as unevaluated FP32 pairs (2Sum: the sum's
+//     rounding errors are carried along, about 48 significant bits) and become FP64 once per
+//     column; a sum that leaves the finite FP32 range is formed again in FP64;
+//   * the FP64 divisions and the N^2 rank comparisons are spread over the cluster's SMs.
+#include <cuda.h>
+#include <cuda_runtime.h>
+
+#include "device.cuh"
+#include "internal.h"
+
+namespace pidk {
+
+namespace {
+
+constexpr int kFinCtas = 8;        // CTAs per ensemble: the portable cluster size
+constexpr int kFinThreads = 512;
+constexpr int kFinWarps = kFinThreads / 32;
+constexpr int kFinMaxN = 512;
+constexpr int kFinMaxRows = kFinMaxN / kFinCtas;       // members per CTA
+constexpr int kFinRowsPerWarp = kFinMaxRows / kFinWarps;
+constexpr float kInf = 3.402823466e38f;                // largest finite FP32
+
+__device__ __forceinline__ const FinDesc& fin_desc(const FinParams& p, int e) {
+  return p.descs ? p.descs[e] : p.one;
+}
+
+// hi + lo += x, with the rounding error of the FP32 addition kept in lo (2Sum, Knuth).
+__device__ __forceinline__ void pair_add(float2& s, float x) {
+  const float t = s.x + x;
+  const float b = t - s.x;
+  s.y += (s.x - (t - b)) + (x - b);
+  s.x = t;
+}
+__device__ __forceinline__ void pair_add(float2& s, float2 v) {
+  pair_add(s, v.x);
+  s.y += v.y;
+}
+
+// State shared by the members of one CTA.
+struct FinShared {
+  float2 acc[kFinThreads];              // partial column sums
+  double tot[2 * kFinMaxRows];          // m of this CTA's members, then N A (or B)
+  double csum[kFinCtas];                // every CTA's share of the mean contour's mass
+  unsigned long long key[kFinMaxN];     // order keys of all depths
+};
+
+// Members of one CTA: [m0, m0 + nm), and cp = the power of two that holds ceil(N / CTAs).
+struct FinSpan {
+  int N, m0, nm, cp;
+};
+__device__ __forceinline__ FinSpan fin_span(int N, int rank) {
+  FinSpan s;
+  const int per = (N + kFinCtas - 1) / kFinCtas;
+  s.N = N;
+  s.m0 = min(N, rank * per);
+  s.nm = min(N, s.m0 + per) - s.m0;
+  s.cp = 1;
+  while (s.cp < per) s.cp *= 2;
+  return s;
+}
+
+// Columns of the [rows][2N] partials that belong to this CTA's members into sh.tot: m and
+// N A, or (second) the second half alone. Thread t takes the rows t / columns, + T / columns,
+// ... of one column; the order depends on N and rows alone.
+__device__ void fin_reduce(FinShared& sh, const float* part, int rows, const FinSpan& sp, bool second) {
+  const int ncol = second ? sp.cp : 2 * sp.cp;
+  const int RG = kFinThreads / ncol;
+  const int t = threadIdx.x;
+  const int64_t stride = 2 * static_cast<int64_t>(sp.N);
+  {
+    const int col = t & (ncol - 1), rg = t / ncol;
+    const int lm = col & (sp.cp - 1);
+    const int half = (second || col >= sp.cp) ? 1 : 0;
+    float2 s = make_float2(0.f, 0.f);
+    if (lm < sp.nm) {
+      const float* src = part + half * sp.N + sp.m0 + lm;
+      int r = rg;
+      for (; r + 7 * RG < rows; r += 8 * RG) {   // 8 loads in flight
+        float v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = __ldcg(src + (r + k * RG) * stride);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) pair_add(s, v[k]);
+      }
+      float v[7];
+#pragma unroll
+      for (int k = 0; k < 7; ++k) v[k] = r + k * RG < rows ? __ldcg(src + (r + k * RG) * stride) : 0.f;
+#pragma unroll
+      for (int k = 0; k < 7; ++k) pair_add(s, v[k]);
+    }
+    sh.acc[t] = s;
+  }
+  __syncthreads();
+  {
+    const int L = min(32, RG);           // lanes that share one column
+    const int c = t / L, l = t & (L - 1);
+    float2 s = make_float2(0.f, 0.f);
+    if (c < ncol)
+      for (int k = l; k < RG; k += L) pair_add(s, sh.acc[k * ncol + c]);
+    for (int o = L / 2; o > 0; o >>= 1) {
+      const float hi = __shfl_xor_sync(0xffffffffu, s.x, o), lo = __shfl_xor_sync(0xffffffffu, s.y, o);
+      // the larger lane index adds the smaller one's value to its own or the other way round:
+      // both lanes form the same sum because the lower lane's pair always comes first
+      const float2 other = make_float2(hi, lo);
+      float2 a = (l & o) ? other : s;
+      pair_add(a, (l & o) ? s : other);
+      s = a;
+    }
+    if (c < ncol && l == 0) {
+      double v = static_cast<double>(s.x) + static_cast<double>(s.y);
+      if (!(fabsf(s.x) <= kInf)) {       // infinities, NaN, or beyond the FP32 range: in FP64
+        const int lm = c & (sp.cp - 1), half = (second || c >= sp.cp) ? 1 : 0;
+        v = 0.0;
+        if (lm < sp.nm)
+          for (int r = 0; r < rows; ++r)
+            v += static_cast<double>(__ldcg(part + half * sp.N + sp.m0 + lm + r * stride));
+      }
+      sh.tot[second ? kFinMaxRows + c : (c >= sp.cp ? kFinMaxRows + c - sp.cp : c)] = v;
+    }
+  }
+  __syncthreads();
+}
+
+// The sum of x over all members: every CTA sums its own (xor tree over 64 slots), pushes the
+// result to all CTAs; the cluster barrier that must follow makes csum readable.
+__device__ __forceinline__ void fin_push_sum(FinShared& sh, double x_lo, double x_hi, int rank) {
+  if (threadIdx.x < 32) {
+    const double s = warp_sum(x_lo + x_hi);
+    if (threadIdx.x < kFinCtas) st_cluster(cluster_addr(&sh.csum[rank], threadIdx.x), s);
+  }
+}
+__device__ __forceinline__ double fin_total(const FinShared& sh) {
+  static_assert(kFinCtas == 8, "pairwise sum of eight");
+  return ((sh.csum[0] + sh.csum[1]) + (sh.csum[2] + sh.csum[3])) +
+         ((sh.csum[4] + sh.csum[5]) + (sh.csum[6] + sh.csum[7]));
+}
+
+// Order key of a depth (order_key, with the addition that folds -0 and quietens NaN only
+// where it matters: FP64 additions are slow).
+__device__ __forceinline__ unsigned long long fin_key(double d) {
+  const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(d));
+  const unsigned long long mag = b & 0x7fffffffffffffffull;
+  if (mag == 0 || mag > 0x7ff0000000000000ull) return order_key(d);
+  return (b >> 63) ? ~b : b | 0x8000000000000000ull;
+}
+
+__device__ __forceinline__ void fin_push_key(FinShared& sh, int i, double depth) {
+  const unsigned long long k = fin_key(depth);
+#pragma unroll
+  for (int r = 0; r < kFinCtas; ++r) st_cluster(cluster_addr(&sh.key[i], r), k);
+}
+
+// Ranks of this CTA's members: one warp per member counts the members that are deeper, or as
+// deep with a lower index.
+__device__ __forceinline__ void fin_ranks(const FinShared& sh, const FinSpan& sp, int32_t* rank) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int r = warp; r < sp.nm; r += kFinWarps) {
+    const int i = sp.m0 + r;
+    const unsigned long long ki = sh.key[i];
+    int n = 0;
+    for (int j = lane; j < sp.N; j += 32) {
+      const unsigned long long kj = sh.key[j];
+      n += (kj > ki) || (kj == ki && j < i);
+    }
+    n = __reduce_add_sync(0xffffffffu, n);
+    if (lane == 0) rank[i] = n;
+  }
+}
+
+}  // namespace
+
+// PID-mean, exact full PID and the weighted mean contour. Measured on one GB300 (ncu, device
+// time) against one CTA of 1024 threads in FP64 with a ticket: see the table in DESIGN.
+__global__ void __cluster_dims__(kFinCtas, 1, 1) __launch_bounds__(kFinThreads, 1)
+finalize_kernel(const __grid_constant__ FinParams p) {
+  __shared__ FinShared sh;
+  cluster_arrive();                      // every CTA has started before its memory is written
+  grid_dependency_wait();
+  const FinDesc& d = fin_desc(p, blockIdx.y);
+  const int rank = static_cast<int>(blockIdx.x);
+  const FinSpan sp = fin_span(d.N, rank);
+  const int N = sp.N, t = threadIdx.x;
+  const int kind = d.kind;
+  const bool wm = kind == FIN_WMEAN, second = kind == FIN_LIN2;
+  fin_reduce(sh, d.part, d.n_chunks, sp, second);
+  const int i = sp.m0 + t;
+  const bool mine = t < sp.nm;
+  double m = 0.0, A = 0.0;               // m_i, N A_i (against a weighted mean contour: A_i)
+  if (mine) {
+    m = second ? __ldcg(d.sums + i) : sh.tot[t];
+    A = second ? __ldcg(d.sums + N + i) : sh.tot[kFinMaxRows + t];
+  }
+  cluster_wait();
+  const bool need_mean = !second && (kind != FIN_LIN1 || d.mean_depth != nullptr);
+  double msum = 0.0;
+  if (need_mean) {
+    double lo = 0.0, hi = 0.0;
+    if (t < 32) {
+      if (t < sp.nm) lo = wm ? sh.tot[t] * static_cast<double>(__ldcg(d.coef + sp.m0 + t)) : sh.tot[t];
+      if (t + 32 < sp.nm)
+        hi = wm ? sh.tot[t + 32] * static_cast<double>(__ldcg(d.coef + sp.m0 + t + 32)) : sh.tot[t + 32];
+    }
+    fin_push_sum(sh, lo, hi, rank);
+    cluster_sync_all();
+    if (mine) msum = fin_total(sh);
+  }
+  double depth = 0.0;
+  if (mine) {
+    // The kernels sum A_i against the column sum N u_bar, so in_in = N A_i / (N m_i) (Eq. 17)
+    // and, the mean contour's mass being (1/N) sum_j m_j, mean_out = N A_i / sum_j m_j (Eq. 16).
+    const double in_in = m > 0.0 ? A / (wm ? m : m * N) : 0.0;
+    double mean_out = 0.0;
+    if (need_mean) {
+      mean_out = msum > 0.0 ? A / msum : 0.0;
+      if (d.mean_depth) d.mean_depth[i] = fmin(in_in, mean_out);
+    }
+    if (d.mass) d.mass[i] = m;
+    if (kind == FIN_LIN1) {
+      d.sums[i] = m;                     // the second pass's finalisation reads both
+      d.sums[N + i] = A;
+      d.coef[i] = m > 0.0 ? static_cast<float>(1.0 / (static_cast<double>(N) * m)) : 0.0f;
+    } else {
+      const double in_out = second ? sh.tot[kFinMaxRows + t] : mean_out;
+      depth = fmin(in_in, in_out);
+      if (d.depth) d.depth[i] = depth;
+      if (d.in_in) d.in_in[i] = in_in;
+      if (d.in_out) d.in_out[i] = in_out;
+    }
+  }
+  if (kind != FIN_LIN1 && d.rank != nullptr) {
+    if (mine) fin_push_key(sh, i, depth);
+    cluster_sync_all();
+    fin_ranks(sh, sp, d.rank);
+  }
+}
+
+// ---------------------------------------------------------------------------------------
+// Finalisation of the tensor-core Gram
+// ---------------------------------------------------------------------------------------
+
+namespace {
+
+// acc + comp carries the running sum; comp holds the low-order part lost by acc (Kahan).
+__device__ __forceinline__ void kahan_add(float& acc, float& comp, float v) {
+  const float y = v - comp;
+  const float t = acc + y;
+  comp = (t - acc) - y;
+  acc = t;
+}
+
+// Element `col` of the [n][NN] Gram partials summed over the chunks in order: compensated
+// FP32, close to an FP64 sum at the FP32 rate. 16 values are loaded before they are added.
+__device__ __forceinline__ float gram_chunk_sum(const float* src, int n, int64_t NN) {
+  float acc = 0.f, comp = 0.f;
+  int r = 0;
+  for (; r + 16 <= n; r += 16) {
+    float v[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) v[k] = __ldcs(src + (r + k) * NN);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) kahan_add(acc, comp, v[k]);
+  }
+  for (; r + 4 <= n; r += 4) {
+    float v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = __ldcs(src + (r + k) * NN);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) kahan_add(acc, comp, v[k]);
+  }
+  for (; r < n; ++r) kahan_add(acc, comp, __ldcs(src + r * NN));
+  return acc;
+}
+
+constexpr int kGramSumThreads = 256;
+
+__device__ __forceinline__ float* fin_gram(const FinDesc& d) { return reinterpret_cast<float*>(d.sums + 4 * d.N); }
+
+// Dot products of this warp's rows (warp, warp + 16, ...) of the CTA's [nm][stride] block
+// with the shared vector v: lane l takes the columns l, l + 32, ... in order, then a fixed
+// xor tree.
+__device__ __forceinline__ void rows_dot(const float* C, int stride, int nm, const float* v, int N,
+                                         float (&acc)[kFinRowsPerWarp]) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+  for (int k = 0; k < kFinRowsPerWarp; ++k) acc[k] = 0.f;
+#pragma unroll 4
+  for (int j = lane; j < N; j += 32) {
+    const float vj = v[j];
+#pragma unroll
+    for (int k = 0; k < kFinRowsPerWarp; ++k) {
+      const int r = warp + k * kFinWarps;
+      if (r < nm) acc[k] = fmaf(C[r * stride + j], vj, acc[k]);
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < kFinRowsPerWarp; ++k) acc[k] = warp_sum(acc[k]);
+}
+
+}  // namespace
+
+// The sums of the Gram partials over the chunks, one thread per element (large ensembles).
+// HBM / L2-bound: n_gchunks N^2 floats read once.
+__global__ void __launch_bounds__(kGramSumThreads) gram_sum_kernel(const __grid_constant__ FinParams p) {
+  grid_dependency_wait();
+  grid_launch_dependents();
+  const FinDesc& d = fin_desc(p, blockIdx.y);
+  if (d.gram_inline) return;
+  const int64_t NN = static_cast<int64_t>(d.N) * d.N;
+  const int64_t col = static_cast<int64_t>(blockIdx.x) * kGramSumThreads + threadIdx.x;
+  if (col < NN) fin_gram(d)[col] = gram_chunk_sum(d.gpart + col, d.n_gchunks, NN);
+}
+
+// The calibration of the tensor-core Gram, its depths and ranks.
+//
+// The Gram G' (stored G'[i + j N] ~ G_ij = sum_x w u_i u_j) carries each member's rounding
+// bias in its row and column. Its row sums are known exactly from the same pass:
+// sum_j G_ij = N A_i (the recall identity, Eq. 17). Calibrate by a symmetric diagonal scaling
+// C_ij = d_i d_j (G'_ij + G'_ji) / 2 with d_i sum_j C... = N A_i (symmetric Sinkhorn
+// iteration), then P_ij = C_ij / m_i, IN_in = mean_j P_ij (= A_i / m_i), IN_out = mean_j
+// P_ji. err_est reports the uncalibrated |mean_j G'_ij / m_i - A_i / m_i|. The O(N^2) work runs
+// in FP32 (the scales converge to FP32 precision, ~1e-7, far inside the Gram bound); the
+// per-member scalars are FP64.
+//
+// Each CTA keeps its members' rows of the symmetrised Gram in shared memory (64 x 512 floats at
+// N = 512; rows padded to an odd stride so that the transposed half writes without bank
+// conflicts) and its warps dot them with the scales, which every sweep pushes to all CTAs.
+__global__ void __cluster_dims__(kFinCtas, 1, 1) __launch_bounds__(kFinThreads, 1)
+finalize_gram_kernel(const __grid_constant__ FinParams p) {
+  extern __shared__ float fin_c0[];                     // [nm][N | 1]
+  __shared__ FinShared sh;
+  __shared__ float sd[2][kFinMaxN], sdm[kFinMaxN];      // calibration scales; d_j / m_j
+  __shared__ float starget[kFinMaxRows], sraw[kFinMaxRows];
+  __shared__ int smoved[2][kFinCtas];
+  __shared__ double serr[kFinCtas];
+  cluster_arrive();
+  grid_dependency_wait();
+  grid_launch_dependents();
+  const FinDesc& d = fin_desc(p, blockIdx.y);
+  const int rank = static_cast<int>(blockIdx.x);
+  const FinSpan sp = fin_span(d.N, rank);
+  const int N = sp.N, t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int stride = N | 1;
+  float* const G = fin_gram(d);
+  if (d.gram_inline) {   // sum this CTA's rows of the stored array
+    const int64_t NN = static_cast<int64_t>(N) * N;
+    for (int e = t; e < sp.nm * N; e += kFinThreads) {
+      const int64_t col = static_cast<int64_t>(sp.m0) * N + e;
+      G[col] = gram_chunk_sum(d.gpart + col, d.n_gchunks, NN);
+    }
+  }
+  fin_reduce(sh, d.part, d.n_chunks, sp, false);
+  const int i = sp.m0 + t;
+  const bool mine = t < sp.nm;
+  const double m = mine ? sh.tot[t] : 0.0, A = mine ? sh.tot[kFinMaxRows + t] : 0.0;   // m_i, N A_i
+  cluster_wait();
+  {
+    double lo = 0.0, hi = 0.0;
+    if (t < 32) {
+      if (t < sp.nm) lo = sh.tot[t];
+      if (t + 32 < sp.nm) hi = sh.tot[t + 32];
+    }
+    fin_push_sum(sh, lo, hi, rank);
+  }
+  cluster_sync_all();    // the other CTAs' shares of the mass; their rows of G (inline sums)
+
+  // Row r of the stored array is G'_{., r}, which equals row r of G' up to the rounding of the
+  // tensor-core sums: its raw sum, and one half of C0.
+  for (int r = warp; r < sp.nm; r += kFinWarps) {
+    const float* row = G + static_cast<int64_t>(sp.m0 + r) * N;
+    float acc = 0.f;
+    for (int b = 0; b < N; b += 256) {
+      float x[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const int j = b + lane + 32 * k;
+        x[k] = j < N ? __ldcg(row + j) : 0.f;
+      }
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const int j = b + lane + 32 * k;
+        if (j < N) {
+          acc += x[k];
+          fin_c0[r * stride + j] = x[k];
+        }
+      }
+    }
+    acc = warp_sum(acc);
+    if (lane == 0) sraw[r] = acc;
+  }
+  __syncthreads();
+  {   // ... plus the other half, read across the rows of the other members
+    const int rr = t & (sp.cp - 1), c0 = t / sp.cp, step = kFinThreads / sp.cp;
+    if (rr < sp.nm) {
+      const float* src = G + sp.m0 + rr;
+      for (int c = c0; c < N; c += 8 * step) {
+        float x[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const int cc = c + k * step;
+          x[k] = cc < N ? __ldcg(src + static_cast<int64_t>(cc) * N) : 0.f;
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const int cc = c + k * step;
+          if (cc < N) fin_c0[rr * stride + cc] = 0.5f * (x[k] + fin_c0[rr * stride + cc]);
+        }
+      }
+    }
+  }
+  double in_in = 0.0, err = 0.0;
+  if (mine) {
+    const double msum = fin_total(sh);
+    const double nm_i = m * N;
+    in_in = m > 0.0 ? A / nm_i : 0.0;
+    if (d.mean_depth) d.mean_depth[i] = fmin(in_in, msum > 0.0 ? A / msum : 0.0);
+    if (d.mass) d.mass[i] = m;
+    const double raw = sraw[t];
+    if (d.err_est) err = m > 0.0 ? fabs(raw / nm_i - in_in) : 0.0;
+    starget[t] = static_cast<float>(A);                 // row-sum target N A_i
+    const float s0 = (A > 0.0 && raw > 0.0) ? 1.0f : 0.0f;
+#pragma unroll
+    for (int r = 0; r < kFinCtas; ++r) st_cluster(cluster_addr(&sd[0][i], r), s0);
+  }
+  cluster_sync_all();
+  // Symmetric Sinkhorn: d_r <- sqrt(d_r N A_r / sum_j C0_rj d_j), until no scale moves by more
+  // than 2^-22 relative (at most 24 sweeps).
+  int cur = 0;
+  for (int it = 0; it < 24; ++it) {
+    float acc[kFinRowsPerWarp];
+    rows_dot(fin_c0, stride, sp.nm, sd[cur], N, acc);
+    bool moved = false;
+#pragma unroll
+    for (int k = 0; k < kFinRowsPerWarp; ++k) {
+      const int r = warp + k * kFinWarps;
+      if (r < sp.nm) {
+        const float so = sd[cur][sp.m0 + r];
+        const float sn = (so > 0.f && acc[k] > 0.f) ? sqrtf(so * starget[r] / acc[k]) : 0.f;
+        moved = moved || fabsf(sn - so) > 2.4e-7f * so;
+        if (lane < kFinCtas) st_cluster(cluster_addr(&sd[cur ^ 1][sp.m0 + r], lane), sn);
+      }
+    }
+    const int any = __syncthreads_or(moved);
+    if (t < kFinCtas) st_cluster(cluster_addr(&smoved[cur][rank], t), any);
+    cluster_sync_all();
+    int more = 0;
+#pragma unroll
+    for (int r = 0; r < kFinCtas; ++r) more |= smoved[cur][r];
+    cur ^= 1;
+    if (!more) break;
+  }
+  // IN_out(i) = (1/N) sum_j C_ji / m_j = (d_i / N) sum_j (d_j / m_j) C0_ij (C0 symmetric).
+  double inv_m = 0.0;
+  if (mine) {
+    const float dm = m > 0.0 ? static_cast<float>(static_cast<double>(sd[cur][i]) / m) : 0.f;
+#pragma unroll
+    for (int r = 0; r < kFinCtas; ++r) st_cluster(cluster_addr(&sdm[i], r), dm);
+    if (d.P) inv_m = m > 0.0 ? 1.0 / m : 0.0;
+  }
+  cluster_sync_all();
+  {
+    float acc[kFinRowsPerWarp];
+    rows_dot(fin_c0, stride, sp.nm, sdm, N, acc);
+#pragma unroll
+    for (int k = 0; k < kFinRowsPerWarp; ++k) {
+      const int r = warp + k * kFinWarps;
+      if (r < sp.nm && lane == 0) sraw[r] = sd[cur][sp.m0 + r] * acc[k];
+    }
+  }
+  __syncthreads();
+  double depth = 0.0;
+  if (mine) {
+    const double in_out = static_cast<double>(sraw[t]) / N;
+    depth = fmin(in_in, in_out);
+    if (d.depth) d.depth[i] = depth;
+    if (d.in_in) d.in_in[i] = in_in;
+    if (d.in_out) d.in_out[i] = in_out;
+    if (d.rank) fin_push_key(sh, i, depth);
+    if (d.P) sh.tot[t] = inv_m;          // 1 / m_i: m is in the owner's registers by now
+  }
+  if (d.err_est) {
+    double e = 0.0;
+    if (t < kFinMaxRows) {               // the members sit in the first two warps
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) err = fmax(err, __shfl_xor_sync(0xffffffffu, err, o));
+      if (lane == 0) sh.csum[warp] = err;
+    }
+    __syncthreads();
+    if (t == 0) {
+      e = fmax(sh.csum[0], sh.csum[1]);
+      st_cluster(cluster_addr(&serr[rank], 0), e);
+    }
+  }
+  cluster_sync_all();
+  if (d.err_est && rank == 0 && t == 0) {
+    double e = serr[0];
+#pragma unroll
+    for (int r = 1; r < kFinCtas; ++r) e = fmax(e, serr[r]);
+    d.err_est[0] = e;
+  }
+  if (d.rank) fin_ranks(sh, sp, d.rank);
+  if (d.P) {
+    // P[r][c] = C_rc / m_r. Small ensembles: written here; else C (FP32) and 1 / m_r are
+    // stored for gram_matrix_kernel.
+    const bool here = N <= kFinInlineMatrixN;
+    float* const C = G + static_cast<int64_t>(N) * N;
+    for (int r = warp; r < sp.nm; r += kFinWarps) {
+      const float sr = sd[cur][sp.m0 + r];
+      const double inv = sh.tot[r];
+      const int64_t row = static_cast<int64_t>(sp.m0 + r) * N;
+      for (int c = lane; c < N; c += 32) {
+        const float v = sr * sd[cur][c] * fin_c0[r * stride + c];
+        if (here) d.P[row + c] = static_cast<double>(v) * inv;
+        else C[row + c] = v;
+      }
+    }
+    if (!here && mine) d.sums[i] = inv_m;
+  }
+}
+
+// P = C / m per row, over the whole GPU: its N^2 FP64 conversions and products take 17 us on one
+// cluster at N = 512.
+__global__ void __launch_bounds__(256) gram_matrix_kernel(const __grid_constant__ FinParams p) {
+  grid_dependency_wait();
+  const FinDesc& d = fin_desc(p, blockIdx.y);
+  const int N = d.N;
+  if (d.P == nullptr || N <= kFinInlineMatrixN) return;
+  const float* C = fin_gram(d) + static_cast<int64_t>(N) * N;
+  const int NN = N * N;
+  for (int e = blockIdx.x * 256 + threadIdx.x; e < NN; e += gridDim.x * 256)
+    d.P[e] = static_cast<double>(__ldcg(C + e)) * __ldcg(d.sums + e / N);
+}
+
+cudaError_t finalize_kernels_init() {
+  return cudaFuncSetAttribute(finalize_gram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              kFinMaxRows * (kFinMaxN | 1) * static_cast<int>(sizeof(float)));
+}
+
+namespace {
+
+template <typename K>
+cudaError_t fin_launch(K kernel, dim3 grid, int threads, size_t smem, bool pdl, const FinParams& p,
+                       cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(static_cast<unsigned>(threads));
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, p);
+}
+
+}  // namespace
+
+cudaError_t launch_finalize(const FinParams& p, const FinLaunch& l, cudaStream_t s) {
+  const dim3 grid(kFinCtas, static_cast<unsigned>(l.count));
+  if (!l.gram) return fin_launch(finalize_kernel, grid, kFinThreads, 0, l.pdl, p, s);
+  cudaError_t e = cudaSuccess;
+  bool pdl = l.pdl;
+  const unsigned NN = static_cast<unsigned>(l.max_n) * static_cast<unsigned>(l.max_n);
+  if (l.sum_gram) {
+    e = fin_launch(gram_sum_kernel, dim3((NN + kGramSumThreads - 1) / kGramSumThreads, grid.y),
+                   kGramSumThreads, 0, pdl, p, s);
+    if (e != cudaSuccess) return e;
+    pdl = true;
+  }
+  const size_t rows = (static_cast<size_t>(l.max_n) + kFinCtas - 1) / kFinCtas;
+  e = fin_launch(finalize_gram_kernel, grid, kFinThreads, rows * (l.max_n | 1) * sizeof(float), pdl, p, s);
+  if (e != cudaSuccess || !l.matrix) return e;
+  return fin_launch(gram_matrix_kernel, dim3((NN + 1023) / 1024, grid.y), 256, 0, true, p, s);
+}
+
+// ---------------------------------------------------------------------------------------
+// More than 512 members (member-blocked path)
+// ---------------------------------------------------------------------------------------
+
+namespace {
+
+constexpr int kLargeThreads = 1024;
+
+// Column block `cb` of a [rows][cols] array: 32 columns (lanes) x 32 warps over rows;
+// the 32 warp sums are then combined in warp order. Deterministic.
+__device__ void reduce_columns(const float* src, int rows, int cols, int cb, double* dst,
+                               double (*scratch)[33]) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int col = cb * 32 + lane;
+  double acc = 0.0;
+  if (col < cols) {
+#pragma unroll 4
+    for (int r = warp; r < rows; r += 32) acc += static_cast<double>(src[static_cast<size_t>(r) * cols + col]);
+  }
+  scratch[warp][lane] = acc;
+  __syncthreads();
+  if (warp == 0) {
+    double t = 0.0;
+    for (int w = 0; w < 32; ++w) t += scratch[w][lane];
+    if (col < cols) dst[col] = t;
+  }
+  __syncthreads();
+}
+
+}  // namespace
+
+// Reduction and per-member outputs of N > 512 members (no Gram; ranks come from a separate
+// kernel).
+__global__ void __launch_bounds__(kLargeThreads, 1) finalize_large_kernel(const __grid_constant__ FinParams p) {
+  const FinDesc& d = p.one;
+  __shared__ double scratch[32][33];
+  __shared__ double sred[kLargeThreads];
+  __shared__ int is_last;
+  const int N = d.N;
+  const int nb = (2 * N + 31) / 32;
+  const int dst_off = d.kind == FIN_LIN2 ? 2 * N : 0;
+  for (int cb = blockIdx.x; cb < nb; cb += d.slices)
+    reduce_columns(d.part, d.n_chunks, 2 * N, cb, d.sums + dst_off, scratch);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) is_last = (atomicAdd(d.ticket, 1u) == static_cast<unsigned>(d.slices - 1));
+  __syncthreads();
+  if (!is_last) return;
+  __threadfence();
+  const double* S = d.sums;
+  const bool wm = d.kind == FIN_WMEAN;
+  double acc = 0.0;
+  for (int j = threadIdx.x; j < N; j += kLargeThreads)
+    acc += wm ? __ldcg(S + j) * static_cast<double>(__ldg(d.coef + j)) : __ldcg(S + j);
+  sred[threadIdx.x] = acc;
+  __syncthreads();
+  for (int o = kLargeThreads / 2; o > 0; o >>= 1) {
+    if (static_cast<int>(threadIdx.x) < o) sred[threadIdx.x] += sred[threadIdx.x + o];
+    __syncthreads();
+  }
+  const double mbar = wm ? sred[0] : sred[0] / N;
+  for (int j = threadIdx.x; j < N; j += kLargeThreads) {
+    const double m = __ldcg(S + j), A = wm ? __ldcg(S + N + j) : __ldcg(S + N + j) / N;
+    const double in_in = m > 0.0 ? A / m : 0.0;
+    const double mean_out = mbar > 0.0 ? A / mbar : 0.0;
+    if (d.mass) d.mass[j] = m;
+    if (d.mean_depth) d.mean_depth[j] = fmin(in_in, mean_out);
+    if (d.kind == FIN_LIN1) {
+      d.coef[j] = m > 0.0 ? static_cast<float>(1.0 / (static_cast<double>(N) * m)) : 0.0f;
+      continue;
+    }
+    const double in_out = d.kind == FIN_LIN2 ? __ldcg(S + 3 * N + j) : mean_out;
+    if (d.depth) d.depth[j] = fmin(in_in, in_out);
+    if (d.in_in) d.in_in[j] = in_in;
+    if (d.in_out) d.in_out[j] = in_out;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) *d.ticket = 0u;
+}
+
+cudaError_t launch_finalize_large(const FinParams& p, cudaStream_t s) {
+  finalize_large_kernel<<<static_cast<unsigned>(p.one.slices), kLargeThreads, 0, s>>>(p);
+  return cudaGetLastError();
+}
+
+}  // namespace pidk

@@ -74,7 +74,7 @@ pid_status plan_gram(pid_handle h, const EnsInput& in, GramPlan* gp) {
   // Without TMA the FP32 ring is unused: keep one minimal stage.
   gp->stage_floats = gp->tma ? static_cast<int32_t>(rup(in.N * gp->TS + gp->TS, 32)) : 32;
   gp->gpart_bytes = rup(static_cast<int64_t>(gp->n_gchunks) * in.N * in.N * 4, 256);
-  gp->part_bytes = rup(static_cast<int64_t>(gp->n_gchunks) * 2 * in.N * 8, 256);
+  gp->part_bytes = rup(static_cast<int64_t>(gp->n_gchunks) * 2 * in.N * 4, 256);
   gram_geometry(h, gp->G, gp->mpw, gp->wide, gp->prec, gp->stage_floats, &gp->dF, &gp->dO,
                 &gp->smem);
   gp->flops = (in.precision == PID_SPLIT_BF16 ? 3.0 : 1.0) * 2.0 * static_cast<double>(in.N) *
@@ -167,7 +167,7 @@ static pid_status gram_launch(pid_handle h, const GramParams& gpar, int G, int m
   return PID_OK;
 }
 
-pid_status launch_gram_one(pid_handle h, const EnsInput& in, GramPlan& gp, double* part,
+pid_status launch_gram_one(pid_handle h, const EnsInput& in, GramPlan& gp, float* part,
                            float* gpart, float* scale, cudaStream_t s, bool scales_ready) {
   GramParams gpar;
   std::memset(&gpar, 0, sizeof(gpar));

@@ -204,6 +204,7 @@ __global__ void __launch_bounds__(gram_threads<G, EXACT>(), 1) gram_kernel(const
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  grid_launch_dependents();   // the finalisation's CTAs may come up as this grid's leave
   const uint32_t tmem_base = *tmem_slot + static_cast<uint32_t>(grp) * NBUF * BUFC;
   // Each group takes a contiguous run of the flat unit list holding an equal share of the
   // work, so it looks an ensemble's descriptor up once per ensemble it meets.
@@ -705,8 +706,8 @@ __global__ void __launch_bounds__(gram_threads<G, EXACT>(), 1) gram_kernel(const
         const float as = warp_sum(accA[m]);
         const int i = q + m * G;
         if (lane == 0 && i < N) {
-          d.part[static_cast<size_t>(c) * 2 * N + i] = static_cast<double>(ms);
-          d.part[static_cast<size_t>(c) * 2 * N + N + i] = static_cast<double>(as);
+          d.part[static_cast<size_t>(c) * 2 * N + i] = ms;
+          d.part[static_cast<size_t>(c) * 2 * N + N + i] = as;
         }
       }
     }

@@ -158,6 +158,7 @@ __global__ void __launch_bounds__(kTiledThreads, 1) gram_tiled_kernel(const __gr
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  grid_launch_dependents();   // the finalisation's CTAs may come up as this grid's leave
   const uint32_t tmem = *tmem_slot;
   bool ok = true;
 

@@ -50,7 +50,7 @@ struct EnsDesc {  // 64-byte aligned through its CUtensorMap members
   const float* data;    // [N][ld]
   const float* w;       // [M] or nullptr (unit cell measure)
   const float* coef;    // [N] column-sum coefficients c_j; nullptr = 1/N for every member
-  double* part;         // [n_chunks][2N] partial sums: m_i, then N A_i (pass 1) or B_i (pass 2)
+  float* part;          // [n_chunks][2N] FP32 partial sums: m_i, then N A_i (pass 1) or B_i (pass 2)
   int64_t ld;
   int32_t N, M;
   int32_t chunk_cells;  // multiple of the stage width sub*T
@@ -161,8 +161,8 @@ struct TiledParams {
   uint32_t* err;
 };
 
-// Finalisation of one ensemble: fixed-order FP64 reduction of the chunk partials, then
-// inclusion fractions, depth and rank.
+// Finalisation of one ensemble: fixed-order reduction of the chunk partials, then inclusion
+// fractions, depth and rank (finalize.cu; more than 512 members: blocked.cu).
 enum FinKind : int32_t {
   FIN_MEAN = 0,   // PID-mean outputs from (m, A)
   FIN_LIN1 = 1,   // first pass of exact full PID: keep (m, A), emit coefficients 1/(N m_j)
@@ -172,15 +172,15 @@ enum FinKind : int32_t {
 };
 
 struct FinDesc {
-  const double* part;      // [n_chunks][2N]
+  const float* part;       // [n_chunks][2N]
   const float* gpart;      // FIN_GRAM: [n_gchunks][N][N] float32 Gram partials (col-major)
   int32_t N, n_chunks;
   int32_t n_gchunks, kind;
-  int32_t slices;          // CTAs working on this ensemble
-  int32_t pad0;
+  int32_t slices;          // more than 512 members: CTAs working on this ensemble
+  int32_t gram_inline;     // FIN_GRAM: the finalisation sums the Gram partials itself
   double* sums;            // workspace [4N] FP64 m, A, (second-pass m), B; then FP32 G [N*N], C0 [N*N]
   float* coef;             // FIN_LIN1 writes [N] coefficients here; FIN_WMEAN reads c_j
-  unsigned int* ticket;    // zero before the launch; the last CTA resets it
+  unsigned int* ticket;    // more than 512 members: zero before the launch, reset by the last CTA
   double* depth;
   double* in_in;
   double* in_out;
@@ -199,6 +199,16 @@ struct FinParams {
   uint32_t* err;
 };
 
+// What a finalisation launch over several ensembles needs besides the descriptors.
+struct FinLaunch {
+  int count = 0;           // ensembles
+  bool gram = false;       // FIN_GRAM ensembles (else: none of them is)
+  int max_n = 0;           // largest N
+  bool sum_gram = false;   // some ensemble's Gram partials are summed by a launch of their own
+  bool matrix = false;     // some ensemble wants P and its rows by a launch of their own
+  bool pdl = false;        // the kernel before it in the stream is its producer
+};
+
 struct IsoParams {
   const float* F;
   void* U;                 // float32 [N][ld_out], or bfloat16 bit patterns when out_bf16
@@ -208,9 +218,13 @@ struct IsoParams {
   int32_t out_bf16;
 };
 
-// Work items of the finalisation's Gram reduction: 32 warps each sum one 32-column block
-// of the [n_gchunks][N*N] partials, so an item covers 1024 columns.
-constexpr int fin_gram_items(int N) { return (N * N + 1023) / 1024; }
+// The Gram partials of small ensembles are summed by the finalisation's own CTAs (a launch
+// less); above this many bytes a launch over the whole GPU sums them first. 8 CTAs read about
+// 1 TB/s, so 2 MB cost them what the extra launch does.
+inline bool fin_gram_inline(int64_t N, int64_t n_gchunks) { return n_gchunks * N * N * 4 <= (int64_t(2) << 20); }
+// Up to this many members the finalisation writes P itself; above, a launch over the whole
+// GPU does (N^2 FP64 products, at 2 per clock and SM).
+constexpr int kFinInlineMatrixN = 96;
 
 // Launchers (stream.cu).
 // Kernel family of an isovalue mode: 0 none, 1 normal, 2 step (either direction) and the
@@ -219,7 +233,9 @@ inline int iso_kind(int32_t iso_mode) { return iso_mode == ISO_NONE ? 0 : (iso_m
 
 cudaError_t launch_stream(const StreamParams& p, int vec, int mpw, int G, int iso_kind, bool coef,
                           int grid, size_t smem, cudaStream_t s);
-cudaError_t launch_finalize(const FinParams& p, int grid_x, int grid_y, cudaStream_t s);
+cudaError_t launch_finalize(const FinParams& p, const FinLaunch& l, cudaStream_t s);   // finalize.cu
+cudaError_t finalize_kernels_init();
+cudaError_t launch_finalize_large(const FinParams& p, cudaStream_t s);   // N > 512
 cudaError_t launch_iso(const IsoParams& p, cudaStream_t s);
 cudaError_t launch_member_coef(const double* r, int64_t N, float* coef, uint32_t* err,
                                cudaStream_t s);

@@ -3,9 +3,9 @@
 // Some callers cannot allocate device memory when they need a depth: real-time loops where
 // a cudaMalloc would synchronise the device, and host applications that hand out all
 // device memory through their own allocator. The regular entry points allocate workspace through
-// a handle; this one keeps its scratch (the per-chunk partial sums, the FP64 totals, the
-// finalisation ticket and the device error word) in a fixed array compiled into the
-// library, and otherwise runs the same streaming and finalisation kernels as pid_mean.
+// a handle; this one keeps its scratch (the per-chunk partial sums, the FP64 totals and the
+// device error word) in a fixed array compiled into the library, and otherwise runs the same
+// streaming and finalisation kernels as pid_mean.
 #include <cuda_runtime.h>
 
 #include <cstring>
@@ -20,7 +20,7 @@ namespace {
 
 // 4 MiB per device, held by every GPU that loads the library until the process exits.
 constexpr size_t kScratchBytes = size_t(4) << 20;
-constexpr size_t kHeaderBytes = 256;  // [0] error word, [1] finalisation ticket (uint32)
+constexpr size_t kHeaderBytes = 256;  // [0] error word (uint32)
 
 __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
@@ -81,18 +81,18 @@ extern "C" pid_status pid_mean_noalloc(const float* U, int64_t N, int64_t M, int
   pidh::EnsPlan pl;
   if ((st = pidh::plan_stream(&ctx, in, &pl)) != PID_OK) return st;
 
-  // Scratch layout: header | FP64 totals [4N] | per-chunk partials [n_chunks][2N].
+  // Scratch layout: header | FP64 totals [4N] | per-chunk partials [n_chunks][2N] (sized, as
+  // documented, for 8 bytes each).
   const size_t sums_bytes = (static_cast<size_t>(4 * N) * 8 + 255) / 256 * 256;
   const size_t part_bytes = static_cast<size_t>(pl.desc.n_chunks) * 2 * N * 8;
   if (kHeaderBytes + sums_bytes + part_bytes > kScratchBytes) return PID_ERR_UNSUPPORTED;
   char* base = ds->scratch;
   uint32_t* err_word = reinterpret_cast<uint32_t*>(base);
-  unsigned int* ticket = reinterpret_cast<unsigned int*>(base) + 1;
   double* sums = reinterpret_cast<double*>(base + kHeaderBytes);
-  double* part = reinterpret_cast<double*>(base + kHeaderBytes + sums_bytes);
+  float* part = reinterpret_cast<float*>(base + kHeaderBytes + sums_bytes);
 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  // The array keeps the previous call's contents: the error word and ticket must start at 0.
+  // The array keeps the previous call's contents: the error word must start at 0.
   if (cudaMemsetAsync(base, 0, kHeaderBytes, s) != cudaSuccess) return PID_ERR_CUDA;
 
   StreamParams sp;
@@ -131,16 +131,16 @@ extern "C" pid_status pid_mean_noalloc(const float* U, int64_t N, int64_t M, int
   fd.n_chunks = pl.desc.n_chunks;
   fd.kind = FIN_MEAN;
   fd.sums = sums;
-  fd.ticket = ticket;
   fd.depth = depth;
   fd.in_in = in_in;
   fd.in_out = in_out;
   fd.rank = rank;
-  const int nb = (2 * fd.N + 31) / 32;
-  fd.slices = nb < 1 ? 1 : (nb > 2 * ds->sms ? 2 * ds->sms : nb);
   fp.n_ens = 1;
   fp.err = err_word;
-  if (launch_finalize(fp, fd.slices, 1, s) != cudaSuccess) return PID_ERR_CUDA;
+  FinLaunch fl;
+  pidh::fin_launch_add(&fl, fd);
+  fl.pdl = true;
+  if (launch_finalize(fp, fl, s) != cudaSuccess) return PID_ERR_CUDA;
   if (device_status &&
       cudaMemcpyAsync(device_status, err_word, sizeof(uint32_t), cudaMemcpyDeviceToDevice, s) !=
           cudaSuccess)

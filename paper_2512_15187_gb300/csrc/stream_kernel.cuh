@@ -301,6 +301,7 @@ stream_kernel(const __grid_constant__ StreamParams p) {
   // leave together (the other parity belongs to the neighbouring barrier).
   if (threadIdx.x < 2 * NG) flags[threadIdx.x] = 0;
   __syncthreads();
+  grid_launch_dependents();   // the finalisation's CTAs may come up as this grid's leave
 
   // Each group takes a contiguous run of the flat unit list (an equal share of the work).
   // An ensemble's chunks are consecutive units, so a group looks an ensemble up (and
@@ -797,8 +798,8 @@ stream_kernel(const __grid_constant__ StreamParams p) {
       const float a = warp_sum(accA[k]);
       const int i = q + k * G;
       if (lane == 0 && i < N) {
-        d.part[static_cast<size_t>(c) * 2 * N + i] = static_cast<double>(m);
-        d.part[static_cast<size_t>(c) * 2 * N + N + i] = static_cast<double>(a);
+        d.part[static_cast<size_t>(c) * 2 * N + i] = m;
+        d.part[static_cast<size_t>(c) * 2 * N + N + i] = a;
       }
     }
     if constexpr (MAXU) {
