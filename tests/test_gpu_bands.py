@@ -87,3 +87,23 @@ def test_bands_rejects_bad_arguments(H):
         with pytest.raises(B.PidError) as e:
             H.contour_bands(U, r, tau, frac)
         assert e.value.status == B.PID_ERR_INVALID_ARG
+
+
+# the 16-byte path (aligned rows, enough cells) and one cell per thread; member counts around
+# the unrolled loads and the staged flags; ranks within groups (several members of rank 0)
+@pytest.mark.parametrize("N,M,pad", [(1, 1 << 21, 0), (7, 1 << 21, 0), (9, 1 << 21, 4), (17, 40001, 0),
+                                     (16, 40000, 0), (1030, 500, 2)])
+def test_bands_load_paths(H, N, M, pad):
+    import torch
+    U = np.random.default_rng(N + M).random((N, M), dtype=np.float32)
+    U[0, ::5] = np.nan          # never above a threshold
+    big = torch.zeros((N, M + pad), device="cuda")
+    big[:, :M] = _dev(U)
+    rank = np.random.default_rng(N).permutation(N).astype(np.int32) // 2
+    got = to_np(H.contour_bands(big[:, :M], _dev(rank), 0.3, 0.4))
+    b = U > np.float32(0.3) if float(np.float32(0.3)) <= 0.3 else U >= np.float32(0.3)
+    inner = rank < int(np.ceil(0.4 * N))
+    med = int(np.nonzero(rank == 0)[0][-1])
+    want = (b[inner].any(0) * 1 + (b[inner].all(0) if inner.any() else np.zeros(M, bool)) * 2 +
+            b.any(0) * 4 + b.all(0) * 8 + b[med] * 16)
+    assert np.array_equal(got, want.astype(np.uint8))
