@@ -136,9 +136,9 @@ __device__ __forceinline__ void iso_store4(void* base, int64_t off, const float4
     uint2 v;
     v.x = *reinterpret_cast<const uint32_t*>(&a);
     v.y = *reinterpret_cast<const uint32_t*>(&b);
-    *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(base) + off) = v;
+    __stcs(reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(base) + off), v);
   } else {
-    *reinterpret_cast<float4*>(static_cast<float*>(base) + off) = u;
+    __stcs(reinterpret_cast<float4*>(static_cast<float*>(base) + off), u);
   }
 }
 
@@ -148,55 +148,94 @@ __device__ __forceinline__ void iso_store1(void* base, int64_t off, float u) {
   else static_cast<float*>(base)[off] = u;
 }
 
-template <bool BF16>
-__global__ void __launch_bounds__(256) iso_kernel(const __grid_constant__ IsoParams p) {
-  // vector path: 16-byte aligned input rows, output rows aligned to 4 elements
-  const bool vec = ((p.ld & 3) == 0) && ((p.ld_out & 3) == 0) &&
-                   ((reinterpret_cast<uintptr_t>(p.F) & 15) == 0) &&
-                   ((reinterpret_cast<uintptr_t>(p.U) & (BF16 ? 7 : 15)) == 0);
-  const int64_t per_row = vec ? (p.M + 3) / 4 : p.M;
-  const int64_t total = per_row * p.N;
-  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  for (int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; t < total; t += stride) {
-    const int64_t i = t / per_row;
-    const int64_t j = t - i * per_row;
+constexpr int kIsoThreads = 256;
+constexpr int kIsoUnroll = 4;   // 16-byte loads in flight per thread
+
+template <int KIND>
+__device__ __forceinline__ float4 iso_map4(const float4& f, const IsoParams& p) {
+  if constexpr (KIND == ISO_NORMAL) {   // bitwise four scalar evaluations
+    const float2 a = iso_normal2(make_float2(f.x, f.y), p.iso_mu, p.iso_inv);
+    const float2 b = iso_normal2(make_float2(f.z, f.w), p.iso_mu, p.iso_inv);
+    return make_float4(a.x, a.y, b.x, b.y);
+  } else {
+    return make_float4(iso_value(f.x, p.iso_mode, p.iso_mu, p.iso_inv, p.iso_t),
+                       iso_value(f.y, p.iso_mode, p.iso_mu, p.iso_inv, p.iso_t),
+                       iso_value(f.z, p.iso_mode, p.iso_mu, p.iso_inv, p.iso_t),
+                       iso_value(f.w, p.iso_mode, p.iso_mu, p.iso_inv, p.iso_t));
+  }
+}
+
+// HBM-bound: 4 B read and 4 (2) B written per element. Rows lie along the grid's y axis, so no
+// element divides its index; contiguous ensembles come as one row, whatever M is. VEC: rows
+// aligned for 4-element accesses, four of them in flight per thread; else element by element.
+// 64 fields of 2048^2 cells to FP32: 0.453 -> 0.304 ms (7.1 TB/s) against one element group per
+// grid-stride step with a 64-bit division.
+template <bool BF16, int KIND, bool VEC>
+__global__ void __launch_bounds__(kIsoThreads) iso_kernel(const __grid_constant__ IsoParams p) {
+  constexpr int64_t kTile = static_cast<int64_t>(kIsoThreads) * kIsoUnroll * (VEC ? 4 : 1);
+  const int64_t x0 = blockIdx.x * kTile;
+  for (int64_t i = blockIdx.y; i < p.N; i += gridDim.y) {
     const float* src = p.F + i * p.ld;
     const int64_t row = i * p.ld_out;
-    if (vec) {
-      const int64_t x = j * 4;
-      if (x + 4 <= p.M) {
-        const float4 f = __ldg(reinterpret_cast<const float4*>(src + x));
-        float4 u;
-        u.x = iso_value(f.x, p.iso_mode, p.iso_mu, p.iso_inv, p.iso_t);
-        u.y = iso_value(f.y, p.iso_mode, p.iso_mu, p.iso_inv, p.iso_t);
-        u.z = iso_value(f.z, p.iso_mode, p.iso_mu, p.iso_inv, p.iso_t);
-        u.w = iso_value(f.w, p.iso_mode, p.iso_mu, p.iso_inv, p.iso_t);
-        iso_store4<BF16>(p.U, row + x, u);
-      } else {
-        for (int64_t xx = x; xx < p.M; ++xx)
-          iso_store1<BF16>(p.U, row + xx,
-                           iso_value(__ldg(src + xx), p.iso_mode, p.iso_mu, p.iso_inv, p.iso_t));
+    if constexpr (VEC) {
+      float4 f[kIsoUnroll];
+#pragma unroll
+      for (int u = 0; u < kIsoUnroll; ++u) {
+        const int64_t x = x0 + (static_cast<int64_t>(u) * kIsoThreads + threadIdx.x) * 4;
+        f[u] = x + 4 <= p.M ? __ldcs(reinterpret_cast<const float4*>(src + x)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+#pragma unroll
+      for (int u = 0; u < kIsoUnroll; ++u) {
+        const int64_t x = x0 + (static_cast<int64_t>(u) * kIsoThreads + threadIdx.x) * 4;
+        if (x + 4 <= p.M) {
+          iso_store4<BF16>(p.U, row + x, iso_map4<KIND>(f[u], p));
+        } else {
+          for (int64_t xx = x; xx < p.M; ++xx)
+            iso_store1<BF16>(p.U, row + xx,
+                             iso_value(__ldg(src + xx), p.iso_mode, p.iso_mu, p.iso_inv, p.iso_t));
+        }
       }
     } else {
-      iso_store1<BF16>(p.U, row + j,
-                       iso_value(__ldg(src + j), p.iso_mode, p.iso_mu, p.iso_inv, p.iso_t));
+      float f[kIsoUnroll];
+#pragma unroll
+      for (int u = 0; u < kIsoUnroll; ++u) {
+        const int64_t x = x0 + static_cast<int64_t>(u) * kIsoThreads + threadIdx.x;
+        f[u] = x < p.M ? __ldcs(src + x) : 0.f;
+      }
+#pragma unroll
+      for (int u = 0; u < kIsoUnroll; ++u) {
+        const int64_t x = x0 + static_cast<int64_t>(u) * kIsoThreads + threadIdx.x;
+        if (x < p.M)
+          iso_store1<BF16>(p.U, row + x, iso_value(f[u], p.iso_mode, p.iso_mu, p.iso_inv, p.iso_t));
+      }
     }
   }
 }
 
+template <bool BF16>
+static void iso_launch(const IsoParams& q, cudaStream_t s) {
+  IsoParams p = q;
+  if (p.ld == p.M && p.ld_out == p.M) {   // contiguous: one row of N M elements
+    p.M *= p.N;
+    p.N = 1;
+  }
+  // rows that start on 16 bytes in the input and on 4 elements in the output
+  const bool vec = (p.N == 1 || ((p.ld & 3) == 0 && (p.ld_out & 3) == 0)) &&
+                   (reinterpret_cast<uintptr_t>(p.F) & 15) == 0 &&
+                   (reinterpret_cast<uintptr_t>(p.U) & (BF16 ? 7 : 15)) == 0;
+  const int64_t tile = static_cast<int64_t>(kIsoThreads) * kIsoUnroll * (vec ? 4 : 1);
+  const dim3 grid(static_cast<unsigned>((p.M + tile - 1) / tile),
+                  static_cast<unsigned>(p.N < 65535 ? p.N : 65535));
+  const bool normal = p.iso_mode == ISO_NORMAL;
+  if (normal && vec) iso_kernel<BF16, ISO_NORMAL, true><<<grid, kIsoThreads, 0, s>>>(p);
+  else if (normal) iso_kernel<BF16, ISO_NORMAL, false><<<grid, kIsoThreads, 0, s>>>(p);
+  else if (vec) iso_kernel<BF16, ISO_NONE, true><<<grid, kIsoThreads, 0, s>>>(p);
+  else iso_kernel<BF16, ISO_NONE, false><<<grid, kIsoThreads, 0, s>>>(p);
+}
+
 cudaError_t launch_iso(const IsoParams& p, cudaStream_t s) {
-  int dev = 0, sms = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int64_t work = p.N * ((p.M + 3) / 4);
-  int64_t blocks = (work + 255) / 256;
-  const int64_t cap = static_cast<int64_t>(sms) * 8;
-  if (blocks > cap) blocks = cap;
-  if (blocks < 1) blocks = 1;
-  if (p.out_bf16)
-    iso_kernel<true><<<static_cast<int>(blocks), 256, 0, s>>>(p);
-  else
-    iso_kernel<false><<<static_cast<int>(blocks), 256, 0, s>>>(p);
+  if (p.out_bf16) iso_launch<true>(p, s);
+  else iso_launch<false>(p, s);
   return cudaGetLastError();
 }
 

@@ -244,3 +244,25 @@ def test_soft_masks_bf16(H, kind, sup, sigma, N, Hh, W):
     # bfloat16 keeps 8 significant bits (7 stored): half an ulp is at most 2^-8 of the value
     err = np.abs(b.float().cpu().numpy() - ref)
     assert np.all(err <= np.abs(ref) * 2.0 ** -8 + 1e-6)
+
+
+# contiguous ensembles as one row (any M, tails of 1 to 3 elements), aligned and unaligned
+# strided rows, and an unaligned base, against the FP64 map
+@pytest.mark.parametrize("N,M,ld,off", [(3, 4097, 4097, 0), (5, 4096, 4096, 0), (7, 1001, 1001, 0),
+                                        (3, 4097, 4100, 0), (3, 4097, 4099, 0), (2, 5000, 5000, 1),
+                                        (1, 3, 3, 0)])
+@pytest.mark.parametrize("kind", ["normal", "uniform"])
+def test_soft_mask_store_paths(H, N, M, ld, off, kind):
+    import torch
+    buf = torch.zeros(N * ld + 4, device="cuda")
+    F = buf[off:off + N * ld].view(N, ld)[:, :M]
+    F.copy_(torch.rand((N, M), device="cuda", generator=torch.Generator("cuda").manual_seed(N * M)) * 2 - 0.5)
+    ref = (O.iso_soft_mask if kind == "normal" else O.iso_soft_mask_uniform)(to_np(F), 0.5, 0.2)
+    for cols in (M, M + 3, M + 4):           # output rows with and without room to spare
+        out = torch.full((N, cols), -1.0, device="cuda")
+        H.soft_masks(F, 0.5, 0.2, kind=kind, out=out)
+        H.sync()
+        assert np.max(np.abs(to_np(out[:, :M]) - ref)) <= 5e-7
+        assert (out[:, M:] == -1.0).all()
+        b16 = H.soft_masks(F, 0.5, 0.2, kind=kind, dtype=torch.bfloat16)
+        assert torch.equal(b16, out[:, :M].to(torch.bfloat16))
