@@ -137,30 +137,183 @@ __global__ void __launch_bounds__(256) accum_kernel(const __grid_constant__ Bloc
   }
 }
 
-// rank[i] = #{j : d_j > d_i or (d_j == d_i and j < i)}; depths staged through shared memory.
-// rank[i] += number of members j in this block's slice of [0, N) (blockIdx.y of gridDim.y
-// equal slices) that are deeper than i, or as deep with a lower index. The slices run as
-// separate blocks for occupancy; the counts are integers, so adding them with atomics
+// ---- finalisation: the outputs of Eq. 10 / Eq. 16 from the chunk partials ----
+
+constexpr int kLargeThreads = 256;
+constexpr int kLargeMembers = 32;                          // members per CTA of the reduction
+constexpr int kLargeRows = kLargeThreads / kLargeMembers;  // row groups that share a column
+
+struct LargeFin {
+  const float* part;       // [n_chunks][2N]
+  int64_t N;
+  int32_t n_chunks, kind;  // FinKind (no Gram)
+  double* sums;            // [2N] m, N A of the first pass; [N] B of the second
+  double* block_mass;      // [ceil(N / 32)] mass sums, then their total
+  unsigned int* ticket;    // zero before the launch; the last CTA resets it
+  float* coef;             // FIN_LIN1 writes the coefficients; FIN_WMEAN reads them
+  double *depth, *in_in, *in_out, *mass, *mean_depth;
+};
+
+// Column i of the partials summed over this thread's rows (FP32 pairs, see pair_add).
+__device__ __forceinline__ float2 large_column(const float* src, int64_t stride, int rows, int r0) {
+  float2 s = make_float2(0.f, 0.f);
+  int r = r0;
+  for (; r + 3 * kLargeRows < rows; r += 4 * kLargeRows) {
+    float v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = __ldcg(src + (r + k * kLargeRows) * stride);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) pair_add(s, v[k]);
+  }
+  for (; r < rows; r += kLargeRows) pair_add(s, __ldcg(src + r * stride));
+  return s;
+}
+
+// The sum of a column's row groups in FP64; sums that leave the finite FP32 range again in FP64.
+__device__ __forceinline__ double large_total(const float2 (*acc)[kLargeMembers], int lane,
+                                              const float* src, int64_t stride, int rows) {
+  float2 s = acc[0][lane];
+#pragma unroll
+  for (int g = 1; g < kLargeRows; ++g) pair_add(s, acc[g][lane]);
+  if (fabsf(s.x) <= kMaxFloat) return static_cast<double>(s.x) + static_cast<double>(s.y);
+  double v = 0.0;
+  for (int r = 0; r < rows; ++r) v += static_cast<double>(__ldcg(src + r * stride));
+  return v;
+}
+
+// Member sums over the chunks, and the masses' total: 32 members per CTA, the CTAs' mass sums
+// added by the last CTA in order. (One CTA used to form every member's outputs as well, with
+// FP64 divisions at two operations per clock: 107 us for 10 000 members.)
+__global__ void __launch_bounds__(kLargeThreads) large_sum_kernel(const __grid_constant__ LargeFin p) {
+  __shared__ float2 acc[2][kLargeRows][kLargeMembers];
+  __shared__ double red[kLargeThreads];
+  __shared__ bool last;
+  const int lane = threadIdx.x & 31, rg = threadIdx.x >> 5;
+  const int64_t i = static_cast<int64_t>(blockIdx.x) * kLargeMembers + lane;
+  const int64_t stride = 2 * p.N;
+  const bool second = p.kind == FIN_LIN2, in = i < p.N;
+  const float2 zero = make_float2(0.f, 0.f);
+  acc[0][rg][lane] = in && !second ? large_column(p.part + i, stride, p.n_chunks, rg) : zero;
+  acc[1][rg][lane] = in ? large_column(p.part + p.N + i, stride, p.n_chunks, rg) : zero;
+  __syncthreads();
+  if (second) {
+    if (rg == 0 && in) p.sums[2 * p.N + i] = large_total(acc[1], lane, p.part + p.N + i, stride, p.n_chunks);
+    return;
+  }
+  if (rg == 1 && in) p.sums[p.N + i] = large_total(acc[1], lane, p.part + p.N + i, stride, p.n_chunks);
+  if (rg == 0) {
+    double m = 0.0;
+    if (in) {
+      m = large_total(acc[0], lane, p.part + i, stride, p.n_chunks);
+      p.sums[i] = m;
+      if (p.kind == FIN_WMEAN) m *= static_cast<double>(p.coef[i]);
+    }
+    m = warp_sum(m);
+    if (lane == 0) {
+      p.block_mass[blockIdx.x] = m;
+      __threadfence();
+      last = atomicAdd(p.ticket, 1u) == gridDim.x - 1;
+    }
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  double t = 0.0;
+  for (unsigned k = threadIdx.x; k < gridDim.x; k += kLargeThreads) t += __ldcg(p.block_mass + k);
+  red[threadIdx.x] = t;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    t = red[threadIdx.x];
+    for (int k = 32; k < kLargeThreads; k += 32) t += red[threadIdx.x + k];
+    t = warp_sum(t);
+    if (threadIdx.x == 0) {
+      p.block_mass[gridDim.x] = t;
+      *p.ticket = 0u;
+    }
+  }
+}
+
+__global__ void __launch_bounds__(kLargeThreads) large_out_kernel(const __grid_constant__ LargeFin p, unsigned blocks) {
+  grid_dependency_wait();
+  const int64_t i = static_cast<int64_t>(blockIdx.x) * kLargeThreads + threadIdx.x;
+  if (i >= p.N) return;
+  const bool second = p.kind == FIN_LIN2;
+  const double m = __ldcg(p.sums + i), A = __ldcg(p.sums + p.N + i);
+  if (p.kind == FIN_LIN1)
+    p.coef[i] = m > 0.0 ? static_cast<float>(1.0 / (static_cast<double>(p.N) * m)) : 0.0f;
+  if (p.mass && !second) p.mass[i] = m;
+  if (p.kind == FIN_LIN1 && !p.mean_depth) return;
+  const double in_in = m > 0.0 ? A / (p.kind == FIN_WMEAN ? m : m * static_cast<double>(p.N)) : 0.0;
+  double in_out = 0.0;
+  if (second) {
+    in_out = __ldcg(p.sums + 2 * p.N + i);
+  } else {
+    const double total = __ldcg(p.block_mass + blocks);
+    in_out = total > 0.0 ? A / total : 0.0;
+    if (p.mean_depth) p.mean_depth[i] = fmin(in_in, in_out);
+  }
+  if (p.kind == FIN_LIN1) return;
+  if (p.depth) p.depth[i] = fmin(in_in, in_out);
+  if (p.in_in) p.in_in[i] = in_in;
+  if (p.in_out) p.in_out[i] = in_out;
+}
+
+// rank[i] += number of members j in this block's slice that are deeper than i, or as deep with a
+// lower index. A thread ranks four members against each key it reads from shared memory, and
+// slices that lie wholly below or above the members need no index comparison: about 14
+// instructions per four pairs, and enough slices to fill the GPU (10 000 members: one member
+// per thread and two slices took 141 us; with the finalisation above, 1910 -> 1713 us a call). The counts are integers, so adding them with atomics
 // gives the same ranks in any order. rank must be zero before the launch.
-__global__ void __launch_bounds__(256) rank_kernel(const double* depth, int64_t N, int32_t* rank) {
-  __shared__ unsigned long long tile[2048];   // order keys of the depths
-  const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  const unsigned long long di = order_key(i < N ? depth[i] : 0.0);
-  const int64_t lo = N * blockIdx.y / gridDim.y, hi = N * (blockIdx.y + 1) / gridDim.y;
-  int64_t r = 0;
-  for (int64_t j0 = lo; j0 < hi; j0 += 2048) {
-    const int64_t n = hi - j0 < 2048 ? hi - j0 : 2048;
-    __syncthreads();
-    for (int64_t k = threadIdx.x; k < n; k += blockDim.x) tile[k] = order_key(depth[j0 + k]);
-    __syncthreads();
-    if (i < N) {
-      for (int64_t k = 0; k < n; ++k) {
-        const unsigned long long dj = tile[k];
-        r += (dj > di) || (dj == di && j0 + k < i);
+constexpr int kRankThreads = 256;
+constexpr int kRankPer = 4;
+constexpr int kRankMembers = kRankThreads * kRankPer;
+constexpr int kRankSlice = 256;                        // largest slice: one key per thread
+
+__global__ void __launch_bounds__(kRankThreads) rank_kernel(const double* depth, int64_t N, int32_t slice,
+                                                            int32_t* rank) {
+  __shared__ unsigned long long tile[kRankSlice];   // order keys of the slice's depths
+  const int64_t i0 = static_cast<int64_t>(blockIdx.x) * kRankMembers;
+  const int64_t j0 = static_cast<int64_t>(blockIdx.y) * slice;
+  const int n = static_cast<int>(min(static_cast<int64_t>(slice), N - j0));
+  if (threadIdx.x < n) tile[threadIdx.x] = order_key(depth[j0 + threadIdx.x]);
+  unsigned long long ki[kRankPer];
+  int cnt[kRankPer];
+#pragma unroll
+  for (int k = 0; k < kRankPer; ++k) {
+    const int64_t i = i0 + k * kRankThreads + threadIdx.x;
+    ki[k] = order_key(i < N ? depth[i] : 0.0);
+    cnt[k] = 0;
+  }
+  __syncthreads();
+  if (j0 + n <= i0) {                       // every j below every i: ties count
+#pragma unroll 4
+    for (int j = 0; j < n; ++j) {
+      const unsigned long long kj = tile[j];
+#pragma unroll
+      for (int k = 0; k < kRankPer; ++k) cnt[k] += kj >= ki[k];
+    }
+  } else if (j0 >= i0 + kRankMembers) {     // every j above every i: ties do not
+#pragma unroll 4
+    for (int j = 0; j < n; ++j) {
+      const unsigned long long kj = tile[j];
+#pragma unroll
+      for (int k = 0; k < kRankPer; ++k) cnt[k] += kj > ki[k];
+    }
+  } else {
+    for (int j = 0; j < n; ++j) {
+      const unsigned long long kj = tile[j];
+#pragma unroll
+      for (int k = 0; k < kRankPer; ++k) {
+        const int64_t i = i0 + k * kRankThreads + threadIdx.x;
+        cnt[k] += (kj > ki[k]) || (kj == ki[k] && j0 + j < i);
       }
     }
   }
-  if (i < N && r > 0) atomicAdd(rank + i, static_cast<int32_t>(r));
+#pragma unroll
+  for (int k = 0; k < kRankPer; ++k) {
+    const int64_t i = i0 + k * kRankThreads + threadIdx.x;
+    if (i < N && cnt[k] > 0) atomicAdd(rank + i, cnt[k]);
+  }
 }
 
 }  // namespace pidk
@@ -183,6 +336,27 @@ static pid_status blocked_pass(pid_handle h, const BlockedParams& p, double byte
   return PID_OK;
 }
 
+static pid_status large_fin(pid_handle h, const LargeFin& p, cudaStream_t s) {
+  ProfScope ps(h, PID_KERNEL_FINALIZE, 0.0, 0.0, s);
+  const unsigned blocks = static_cast<unsigned>((p.N + kLargeMembers - 1) / kLargeMembers);
+  large_sum_kernel<<<blocks, kLargeThreads, 0, s>>>(p);
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>((p.N + kLargeThreads - 1) / kLargeThreads));
+    cfg.blockDim = dim3(kLargeThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, large_out_kernel, p, blocks);
+  }
+  if (e != cudaSuccess) return cuda_fail(h, e, "finalize launch");
+  return PID_OK;
+}
+
 pid_status run_blocked(pid_handle h, const EnsInput& in, const EnsOutputs& out, cudaStream_t s) {
   if (in.mode == PID_MODE_FULL && in.precision != PID_FP32)
     return fail(h, PID_ERR_UNSUPPORTED,
@@ -197,7 +371,8 @@ pid_status run_blocked(pid_handle h, const EnsInput& in, const EnsOutputs& out, 
   const size_t S_bytes = rup(static_cast<int64_t>(n_blocks) * ldS * 4, 256);
   const size_t s_bytes = rup(ldS * 4, 256);
   const size_t part_bytes = rup(static_cast<int64_t>(n_chunks) * 2 * N * 4, 256);
-  const size_t sums_bytes = rup(4 * N * 8, 256);
+  const int64_t fin_blocks = (N + kLargeMembers - 1) / kLargeMembers;
+  const size_t sums_bytes = rup((3 * N + fin_blocks + 1) * 8, 256);
   const size_t coef_bytes = rup(N * 4, 256);
   const size_t dtmp_bytes = (out.rank && !out.depth) ? rup(N * 8, 256) : 0;
   pid_status st = ensure_workspace(h, S_bytes + s_bytes + part_bytes + sums_bytes + coef_bytes +
@@ -219,12 +394,13 @@ pid_status run_blocked(pid_handle h, const EnsInput& in, const EnsOutputs& out, 
   iso_fill(in.is_field ? &in.iso : nullptr, &p.iso_mode, &p.iso_mu, &p.iso_inv, &p.iso_t);
   const double bytes = 4.0 * N * M + (in.w ? 4.0 * M : 0.0);
 
-  FinDesc fd;
+  LargeFin fd;
   std::memset(&fd, 0, sizeof(fd));
   fd.part = p.part;
-  fd.N = static_cast<int32_t>(N);
+  fd.N = N;
   fd.n_chunks = n_chunks;
   fd.sums = sums;
+  fd.block_mass = sums + 3 * N;
   fd.coef = coef;
   fd.ticket = h->tickets;
   fd.depth = out.depth ? out.depth : dtmp;
@@ -238,30 +414,32 @@ pid_status run_blocked(pid_handle h, const EnsInput& in, const EnsOutputs& out, 
     p.coef = coef;
     if ((st = blocked_pass(h, p, bytes, s)) != PID_OK) return st;
     fd.kind = FIN_WMEAN;
-    if ((st = launch_fin_one(h, fd, s)) != PID_OK) return st;
+    if ((st = large_fin(h, fd, s)) != PID_OK) return st;
   } else if ((st = blocked_pass(h, p, bytes, s)) != PID_OK) {
     return st;
   } else if (!linear) {
     fd.kind = FIN_MEAN;
-    if ((st = launch_fin_one(h, fd, s)) != PID_OK) return st;
+    if ((st = large_fin(h, fd, s)) != PID_OK) return st;
   } else {
-    FinDesc f1 = fd;
+    LargeFin f1 = fd;
     f1.kind = FIN_LIN1;
-    f1.depth = nullptr; f1.in_in = nullptr; f1.in_out = nullptr; f1.rank = nullptr;
-    if ((st = launch_fin_one(h, f1, s)) != PID_OK) return st;
+    if ((st = large_fin(h, f1, s)) != PID_OK) return st;
     p.coef = coef;
     if ((st = blocked_pass(h, p, bytes, s)) != PID_OK) return st;
-    FinDesc f2 = fd;
+    LargeFin f2 = fd;
     f2.kind = FIN_LIN2;
-    f2.mass = nullptr; f2.mean_depth = nullptr;
-    if ((st = launch_fin_one(h, f2, s)) != PID_OK) return st;
+    if ((st = large_fin(h, f2, s)) != PID_OK) return st;
   }
   if (out.rank) {
-    const unsigned slices = static_cast<unsigned>(N / 4096 < 1 ? 1 : (N / 4096 > 16 ? 16 : N / 4096));
+    // slices of at most 256 keys, shorter ones where the members alone do not give every SM
+    // a few blocks
+    const int64_t groups = (N + kRankMembers - 1) / kRankMembers;
+    int64_t slice = rup((N * groups + 4 * h->sms - 1) / (4 * h->sms), 32);
+    slice = std::max<int64_t>(32, std::min<int64_t>(slice, kRankSlice));
     cudaError_t e = cudaMemsetAsync(out.rank, 0, static_cast<size_t>(N) * sizeof(int32_t), s);
     if (e != cudaSuccess) return cuda_fail(h, e, "rank reset");
-    rank_kernel<<<dim3(static_cast<unsigned>((N + 255) / 256), slices), 256, 0, s>>>(fd.depth, N,
-                                                                                    out.rank);
+    rank_kernel<<<dim3(static_cast<unsigned>(groups), static_cast<unsigned>((N + slice - 1) / slice)),
+                  kRankThreads, 0, s>>>(fd.depth, N, static_cast<int32_t>(slice), out.rank);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(h, e, "rank kernel launch");
   }

@@ -583,11 +583,9 @@ static pid_status launch_stream_one(pid_handle h, EnsPlan& pl, const float* coef
                        static_cast<int64_t>(pl.desc.N) * pl.desc.M, bytes, s);
 }
 
-pid_status launch_fin_one(pid_handle h, FinDesc fd, cudaStream_t s) {
+pid_status launch_fin_one(pid_handle h, const FinDesc& fd, cudaStream_t s) {
   FinParams fp;
   std::memset(&fp, 0, sizeof(fp));
-  const bool large = fd.N > kMaxMembers;
-  if (large) fd.slices = std::max(1, std::min((2 * fd.N + 31) / 32, 2 * h->sms));
   FinLaunch l;
   fin_launch_add(&l, fd);
   l.pdl = true;   // the kernel before it in the stream wrote its partials
@@ -596,7 +594,7 @@ pid_status launch_fin_one(pid_handle h, FinDesc fd, cudaStream_t s) {
   fp.n_ens = 1;
   fp.err = h->err_word;
   ProfScope ps(h, PID_KERNEL_FINALIZE, 0.0, 0.0, s);
-  cudaError_t e = large ? launch_finalize_large(fp, s) : launch_finalize(fp, l, s);
+  cudaError_t e = launch_finalize(fp, l, s);
   if (e != cudaSuccess) return cuda_fail(h, e, "finalize launch");
   return PID_OK;
 }

@@ -176,7 +176,7 @@ pid_status check_shape(pid_handle h, const void* data, int64_t N, int64_t M, int
                        int64_t max_n = kMaxMembers);
 pid_status launch_member_coef_one(pid_handle h, const double* r, int64_t N, float* coef,
                                   cudaStream_t s);
-pid_status launch_fin_one(pid_handle h, pidk::FinDesc fd, cudaStream_t s);
+pid_status launch_fin_one(pid_handle h, const pidk::FinDesc& fd, cudaStream_t s);
 // Counts one ensemble into a finalisation launch.
 inline void fin_launch_add(pidk::FinLaunch* l, const pidk::FinDesc& fd) {
   ++l->count;

@@ -252,11 +252,28 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+constexpr float kMaxFloat = 3.402823466e38f;   // largest finite FP32
+
+// hi + lo += x, with the rounding error of the FP32 addition kept in lo (2Sum, Knuth).
+__device__ __forceinline__ void pair_add(float2& s, float x) {
+  const float t = s.x + x;
+  const float b = t - s.x;
+  s.y += (s.x - (t - b)) + (x - b);
+  s.x = t;
+}
+__device__ __forceinline__ void pair_add(float2& s, float2 v) {
+  pair_add(s, v.x);
+  s.y += v.y;
+}
+
 // Order-preserving integer key of a double: for non-NaN a, b, a < b <=> key(a) < key(b) and
-// a == b <=> key(a) == key(b) (-0 is folded into +0). GB300 issues FP64 compares at a small
-// fraction of the integer rate, so the O(N^2) rank counts compare keys.
+// a == b <=> key(a) == key(b) (-0 is folded into +0). GB300 issues FP64 compares and additions
+// at a small fraction of the integer rate, so the O(N^2) rank counts compare keys, and only
+// zeros and NaN take the addition that folds the sign of zero and quietens NaN.
 __device__ __forceinline__ unsigned long long order_key(double d) {
-  const long long b = __double_as_longlong(d + 0.0);
+  long long b = __double_as_longlong(d);
+  const long long mag = b & 0x7fffffffffffffffll;
+  if (mag == 0 || mag > 0x7ff0000000000000ll) b = __double_as_longlong(d + 0.0);
   return b >= 0 ? static_cast<unsigned long long>(b) | 0x8000000000000000ull
                 : ~static_cast<unsigned long long>(b);
 }

@@ -30,22 +30,9 @@ constexpr int kFinWarps = kFinThreads / 32;
 constexpr int kFinMaxN = 512;
 constexpr int kFinMaxRows = kFinMaxN / kFinCtas;       // members per CTA
 constexpr int kFinRowsPerWarp = kFinMaxRows / kFinWarps;
-constexpr float kInf = 3.402823466e38f;                // largest finite FP32
 
 __device__ __forceinline__ const FinDesc& fin_desc(const FinParams& p, int e) {
   return p.descs ? p.descs[e] : p.one;
-}
-
-// hi + lo += x, with the rounding error of the FP32 addition kept in lo (2Sum, Knuth).
-__device__ __forceinline__ void pair_add(float2& s, float x) {
-  const float t = s.x + x;
-  const float b = t - s.x;
-  s.y += (s.x - (t - b)) + (x - b);
-  s.x = t;
-}
-__device__ __forceinline__ void pair_add(float2& s, float2 v) {
-  pair_add(s, v.x);
-  s.y += v.y;
 }
 
 // State shared by the members of one CTA.
@@ -120,7 +107,7 @@ __device__ void fin_reduce(FinShared& sh, const float* part, int rows, const Fin
     }
     if (c < ncol && l == 0) {
       double v = static_cast<double>(s.x) + static_cast<double>(s.y);
-      if (!(fabsf(s.x) <= kInf)) {       // infinities, NaN, or beyond the FP32 range: in FP64
+      if (!(fabsf(s.x) <= kMaxFloat)) {       // infinities, NaN, or beyond the FP32 range: in FP64
         const int lm = c & (sp.cp - 1), half = (second || c >= sp.cp) ? 1 : 0;
         v = 0.0;
         if (lm < sp.nm)
@@ -147,17 +134,8 @@ __device__ __forceinline__ double fin_total(const FinShared& sh) {
          ((sh.csum[4] + sh.csum[5]) + (sh.csum[6] + sh.csum[7]));
 }
 
-// Order key of a depth (order_key, with the addition that folds -0 and quietens NaN only
-// where it matters: FP64 additions are slow).
-__device__ __forceinline__ unsigned long long fin_key(double d) {
-  const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(d));
-  const unsigned long long mag = b & 0x7fffffffffffffffull;
-  if (mag == 0 || mag > 0x7ff0000000000000ull) return order_key(d);
-  return (b >> 63) ? ~b : b | 0x8000000000000000ull;
-}
-
 __device__ __forceinline__ void fin_push_key(FinShared& sh, int i, double depth) {
-  const unsigned long long k = fin_key(depth);
+  const unsigned long long k = order_key(depth);
 #pragma unroll
   for (int r = 0; r < kFinCtas; ++r) st_cluster(cluster_addr(&sh.key[i], r), k);
 }
@@ -181,8 +159,9 @@ __device__ __forceinline__ void fin_ranks(const FinShared& sh, const FinSpan& sp
 
 }  // namespace
 
-// PID-mean, exact full PID and the weighted mean contour. Measured on one GB300 (ncu, device
-// time) against one CTA of 1024 threads in FP64 with a ticket: see the table in DESIGN.
+// PID-mean, exact full PID and the weighted mean contour. Whole calls against a last CTA that
+// formed the outputs in FP64: 64 x 512^2 fields PID-mean 45.5 -> 33.0 us, 128 x 2^20 exact full
+// PID 215 -> 188 us, of which the finalisation was 15 to 18 us each time.
 __global__ void __cluster_dims__(kFinCtas, 1, 1) __launch_bounds__(kFinThreads, 1)
 finalize_kernel(const __grid_constant__ FinParams p) {
   __shared__ FinShared sh;
@@ -336,6 +315,8 @@ __global__ void __launch_bounds__(kGramSumThreads) gram_sum_kernel(const __grid_
 // Each CTA keeps its members' rows of the symmetrised Gram in shared memory (64 x 512 floats at
 // N = 512; rows padded to an odd stride so that the transposed half writes without bank
 // conflicts) and its warps dot them with the scales, which every sweep pushes to all CTAs.
+// 512 x 2^20 split BF16 with P: the whole call 2806 -> 2411 us against one CTA that did all of
+// this (437 us); the plume step's three items 1076 -> 996 us (131 us).
 __global__ void __cluster_dims__(kFinCtas, 1, 1) __launch_bounds__(kFinThreads, 1)
 finalize_gram_kernel(const __grid_constant__ FinParams p) {
   extern __shared__ float fin_c0[];                     // [nm][N | 1]
@@ -583,91 +564,6 @@ cudaError_t launch_finalize(const FinParams& p, const FinLaunch& l, cudaStream_t
   e = fin_launch(finalize_gram_kernel, grid, kFinThreads, rows * (l.max_n | 1) * sizeof(float), pdl, p, s);
   if (e != cudaSuccess || !l.matrix) return e;
   return fin_launch(gram_matrix_kernel, dim3((NN + 1023) / 1024, grid.y), 256, 0, true, p, s);
-}
-
-// ---------------------------------------------------------------------------------------
-// More than 512 members (member-blocked path)
-// ---------------------------------------------------------------------------------------
-
-namespace {
-
-constexpr int kLargeThreads = 1024;
-
-// Column block `cb` of a [rows][cols] array: 32 columns (lanes) x 32 warps over rows;
-// the 32 warp sums are then combined in warp order. Deterministic.
-__device__ void reduce_columns(const float* src, int rows, int cols, int cb, double* dst,
-                               double (*scratch)[33]) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int col = cb * 32 + lane;
-  double acc = 0.0;
-  if (col < cols) {
-#pragma unroll 4
-    for (int r = warp; r < rows; r += 32) acc += static_cast<double>(src[static_cast<size_t>(r) * cols + col]);
-  }
-  scratch[warp][lane] = acc;
-  __syncthreads();
-  if (warp == 0) {
-    double t = 0.0;
-    for (int w = 0; w < 32; ++w) t += scratch[w][lane];
-    if (col < cols) dst[col] = t;
-  }
-  __syncthreads();
-}
-
-}  // namespace
-
-// Reduction and per-member outputs of N > 512 members (no Gram; ranks come from a separate
-// kernel).
-__global__ void __launch_bounds__(kLargeThreads, 1) finalize_large_kernel(const __grid_constant__ FinParams p) {
-  const FinDesc& d = p.one;
-  __shared__ double scratch[32][33];
-  __shared__ double sred[kLargeThreads];
-  __shared__ int is_last;
-  const int N = d.N;
-  const int nb = (2 * N + 31) / 32;
-  const int dst_off = d.kind == FIN_LIN2 ? 2 * N : 0;
-  for (int cb = blockIdx.x; cb < nb; cb += d.slices)
-    reduce_columns(d.part, d.n_chunks, 2 * N, cb, d.sums + dst_off, scratch);
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) is_last = (atomicAdd(d.ticket, 1u) == static_cast<unsigned>(d.slices - 1));
-  __syncthreads();
-  if (!is_last) return;
-  __threadfence();
-  const double* S = d.sums;
-  const bool wm = d.kind == FIN_WMEAN;
-  double acc = 0.0;
-  for (int j = threadIdx.x; j < N; j += kLargeThreads)
-    acc += wm ? __ldcg(S + j) * static_cast<double>(__ldg(d.coef + j)) : __ldcg(S + j);
-  sred[threadIdx.x] = acc;
-  __syncthreads();
-  for (int o = kLargeThreads / 2; o > 0; o >>= 1) {
-    if (static_cast<int>(threadIdx.x) < o) sred[threadIdx.x] += sred[threadIdx.x + o];
-    __syncthreads();
-  }
-  const double mbar = wm ? sred[0] : sred[0] / N;
-  for (int j = threadIdx.x; j < N; j += kLargeThreads) {
-    const double m = __ldcg(S + j), A = wm ? __ldcg(S + N + j) : __ldcg(S + N + j) / N;
-    const double in_in = m > 0.0 ? A / m : 0.0;
-    const double mean_out = mbar > 0.0 ? A / mbar : 0.0;
-    if (d.mass) d.mass[j] = m;
-    if (d.mean_depth) d.mean_depth[j] = fmin(in_in, mean_out);
-    if (d.kind == FIN_LIN1) {
-      d.coef[j] = m > 0.0 ? static_cast<float>(1.0 / (static_cast<double>(N) * m)) : 0.0f;
-      continue;
-    }
-    const double in_out = d.kind == FIN_LIN2 ? __ldcg(S + 3 * N + j) : mean_out;
-    if (d.depth) d.depth[j] = fmin(in_in, in_out);
-    if (d.in_in) d.in_in[j] = in_in;
-    if (d.in_out) d.in_out[j] = in_out;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) *d.ticket = 0u;
-}
-
-cudaError_t launch_finalize_large(const FinParams& p, cudaStream_t s) {
-  finalize_large_kernel<<<static_cast<unsigned>(p.one.slices), kLargeThreads, 0, s>>>(p);
-  return cudaGetLastError();
 }
 
 }  // namespace pidk

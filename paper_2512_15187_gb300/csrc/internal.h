@@ -162,7 +162,7 @@ struct TiledParams {
 };
 
 // Finalisation of one ensemble: fixed-order reduction of the chunk partials, then inclusion
-// fractions, depth and rank (finalize.cu; more than 512 members: blocked.cu).
+// fractions, depth and rank (finalize.cu; ensembles of more than 512 members: blocked.cu).
 enum FinKind : int32_t {
   FIN_MEAN = 0,   // PID-mean outputs from (m, A)
   FIN_LIN1 = 1,   // first pass of exact full PID: keep (m, A), emit coefficients 1/(N m_j)
@@ -176,11 +176,10 @@ struct FinDesc {
   const float* gpart;      // FIN_GRAM: [n_gchunks][N][N] float32 Gram partials (col-major)
   int32_t N, n_chunks;
   int32_t n_gchunks, kind;
-  int32_t slices;          // more than 512 members: CTAs working on this ensemble
   int32_t gram_inline;     // FIN_GRAM: the finalisation sums the Gram partials itself
+  int32_t pad0;
   double* sums;            // workspace [4N] FP64 m, A, (second-pass m), B; then FP32 G [N*N], C0 [N*N]
   float* coef;             // FIN_LIN1 writes [N] coefficients here; FIN_WMEAN reads c_j
-  unsigned int* ticket;    // more than 512 members: zero before the launch, reset by the last CTA
   double* depth;
   double* in_in;
   double* in_out;
@@ -235,7 +234,6 @@ cudaError_t launch_stream(const StreamParams& p, int vec, int mpw, int G, int is
                           int grid, size_t smem, cudaStream_t s);
 cudaError_t launch_finalize(const FinParams& p, const FinLaunch& l, cudaStream_t s);   // finalize.cu
 cudaError_t finalize_kernels_init();
-cudaError_t launch_finalize_large(const FinParams& p, cudaStream_t s);   // N > 512
 cudaError_t launch_iso(const IsoParams& p, cudaStream_t s);
 cudaError_t launch_member_coef(const double* r, int64_t N, float* coef, uint32_t* err,
                                cudaStream_t s);

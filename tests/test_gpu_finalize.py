@@ -86,3 +86,19 @@ def test_nan_input_reaches_the_outputs(H):
     assert in_in[3] == 0.0 and np.isnan(np.delete(in_in, 3)).all()
     assert (to_np(o["in_out"]) == 0.0).all() and (to_np(o["depth"]) == 0.0).all()
     assert to_np(o["rank"]).tolist() == list(range(20))
+
+
+# beyond the cluster's 512 members: 32 members per CTA of the reduction, rank slices below,
+# above and across the 1024 members of a block, one or several row groups of chunks
+@pytest.mark.parametrize("N,M", [(513, 100), (545, 9001), (1023, 300), (1025, 70000), (2100, 1000)])
+def test_large_ensemble_finalisation(H, N, M):
+    U = synth.random_soft(N, M, seed=N + M, binary_frac=0.3)
+    U[N - 1] = U[0]              # ties across the blocks
+    U[N // 2] = U[0]
+    U[5] = 0.0                   # zero mass
+    Ud = _dev(U)
+    _check(H.mean(Ud), O.pid_mean(U), FP32_TOL)
+    _check(H.full(Ud, mode="linear"), O.pid(U), FP32_TOL)
+    r = np.random.default_rng(N).uniform(0.1, 2.0, N)
+    _check(H.mean_weighted(Ud, _dev(r)), O.pid_mean_weighted(U, r), FP32_TOL)
+    H.sync()
