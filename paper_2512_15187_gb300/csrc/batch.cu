@@ -361,7 +361,7 @@ static pid_status plan_batch(pid_handle h, const pid_ensemble* ens, int count, c
   size_t op_bytes = 0;
   for (int e = 0; e < count; ++e) {
     if (!tiled[e]) continue;
-    fused[e] = store_u && tp[e].prec == PID_BF16 && pl[e].cfg.vec == 1;
+    fused[e] = tp[e].clusters == 0 && store_u && tp[e].prec == PID_BF16 && pl[e].cfg.vec == 1;
     if (fused[e]) {
       op_own[e] = base + off;
       off += align_up(static_cast<int64_t>(tp[e].op_bytes), 1024);

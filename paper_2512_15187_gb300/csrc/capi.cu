@@ -628,7 +628,7 @@ static pid_status run_gram_tiled(pid_handle h, const EnsInput& in, EnsPlan& pl,
   pl.desc.part = part;
   // BF16 operands come straight from the streaming pass (its one-cell-per-lane classes,
   // which every N > 256 uses); split BF16 and E4M3 are staged by their own kernel.
-  const bool fused = tp.prec == PID_BF16 && pl.cfg.vec == 1;
+  const bool fused = tp.clusters == 0 && tp.prec == PID_BF16 && pl.cfg.vec == 1;
   if (fused) {
     pl.desc.op_out = reinterpret_cast<uint16_t*>(ws + off_op);
     pl.desc.op_ld = tp.ldo;
@@ -845,6 +845,7 @@ pid_status pid_create(pid_handle* out, int device, size_t hbm_budget_bytes) {
   h->max_smem = max_smem;
   e = stream_kernels_init(max_smem);
   if (e == cudaSuccess && h->cc >= 100) e = gram_kernels_init(max_smem);
+  for (int R = 3; R <= 4 && e == cudaSuccess && h->cc >= 100; ++R) e = gram_max_clusters(R, &h->gram_clusters[R - 3]);
   if (e != cudaSuccess) {
     cudaGetLastError();
     delete h;

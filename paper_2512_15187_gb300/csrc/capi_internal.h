@@ -50,6 +50,7 @@ struct pid_handle_s {
   int sms = 148;
   int cc = 0;
   int max_smem = 0;
+  int gram_clusters[2] = {0, 0};   // clusters of the cluster Gram that run at once (3 and 4 row blocks)
   size_t budget = 0;
   void* ws = nullptr;          // growable workspace
   size_t ws_bytes = 0;
@@ -142,6 +143,7 @@ struct TiledPlan {
   int prec = 0;            // PID_BF16, PID_SPLIT_BF16 or PID_FP8
   int R = 0;               // 128-row blocks
   int tiles = 0;           // tiles per chunk (gram_tiles)
+  int clusters = 0;        // > 0: one pass by that many clusters (gram_cluster.cu)
   pidk::TileDesc tile[pidk::kMaxTiles];
   int slots = 0;           // 128-row blocks per stage and plane
   int64_t ldo = 0;         // operand row stride in elements (a multiple of 64)

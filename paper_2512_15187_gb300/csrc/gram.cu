@@ -227,6 +227,8 @@ pid_status launch_gram_batch(pid_handle h, const GramPlan& gp, const EnsDesc* de
 // Row-block-tiled Gram (256 < N <= 512)
 // ---------------------------------------------------------------------------------------
 
+constexpr int kClusterMinChunks = 28;
+
 pid_status plan_gram_tiled(pid_handle h, const EnsInput& in, TiledPlan* tp) {
   *tp = TiledPlan{};
   if (in.N > kGramTiledMaxN)
@@ -251,13 +253,19 @@ pid_status plan_gram_tiled(pid_handle h, const EnsInput& in, TiledPlan* tp) {
   chunk = std::min<int64_t>(std::max<int64_t>(chunk, 4096), 65536);
   tp->chunk_cells = chunk;
   tp->n_gchunks = static_cast<int>((in.M + chunk - 1) / chunk);
+  // One pass by clusters once there are chunks for most of them (kClusterMinChunks): a chunk keeps
+  // one cluster of 3 or 4 SMs busy, a chunk's tiles 2 to 6 SMs. Whole calls, tiles -> clusters: split
+  // BF16 300 x 131 072 (32 chunks) 255 -> 208 us, 512 x 1 048 576 2335 -> 1545; but 448 x 100 003
+  // (25 chunks) 294 -> 297, 512 x 5000 (2 chunks) 199 -> 264, BF16 333 x 100 001 (25 chunks) 197 -> 219.
+  const int clusters = h->gram_clusters[tp->R - 3];
+  if (tp->n_gchunks >= kClusterMinChunks) tp->clusters = std::min(clusters, tp->n_gchunks);
   const size_t cap = static_cast<size_t>(h->max_smem > 0 ? h->max_smem : 232448);
   tp->stages = 6;
   while (tp->stages > 2 && gram_tiled_smem_bytes(tp->prec, tp->slots, tp->stages) > cap) --tp->stages;
   tp->smem = gram_tiled_smem_bytes(tp->prec, tp->slots, tp->stages);
   if (tp->smem > cap) return fail(h, PID_ERR_UNSUPPORTED, "tiled Gram stages do not fit shared memory");
   const int64_t plane = rup(static_cast<int64_t>(in.N) * tp->ldo * tp->elem_bytes, 1024);
-  tp->op_bytes = static_cast<size_t>(tp->planes * plane);
+  tp->op_bytes = tp->clusters > 0 ? (in.w ? rup(in.M, 128) * 4 : 0) : static_cast<size_t>(tp->planes * plane);
   tp->gpart_bytes = rup(static_cast<int64_t>(tp->n_gchunks) * in.N * in.N * 4, 256);
   const double nm = static_cast<double>(in.N) * in.M;
   tp->op_rw_bytes = 4.0 * nm + (in.w ? 4.0 * in.M : 0.0) + nm * tp->elem_bytes * tp->planes;
@@ -279,6 +287,30 @@ pid_status launch_gram_tiled_one(pid_handle h, const EnsInput& in, const TiledPl
       if (st != PID_OK) return st;
     }
     op_scale = scale;
+  }
+  if (tp.clusters > 0) {
+    ClusterGramParams cp;
+    std::memset(&cp, 0, sizeof(cp));
+    cp.F = in.data;
+    float* const sqrt_w = in.w ? static_cast<float*>(op) : nullptr;
+    cp.sqrt_w = sqrt_w;
+    cp.gpart = gpart;
+    cp.op_scale = op_scale;
+    cp.ld = in.ld;
+    cp.N = static_cast<int32_t>(in.N);
+    cp.M = static_cast<int32_t>(in.M);
+    cp.R = tp.R;
+    cp.chunk_cells = static_cast<int32_t>(tp.chunk_cells);
+    cp.n_chunks = tp.n_gchunks;
+    cp.stages = gram_cluster_stages(tp.R, tp.prec);
+    cp.vec_ok = in.ld % 4 == 0 && reinterpret_cast<uintptr_t>(in.data) % 16 == 0;
+    iso_fill(in.is_field ? &in.iso : nullptr, &cp.iso_mode, &cp.iso_mu, &cp.iso_inv, &cp.iso_t);
+    cp.err = h->err_word;
+    cp.flags = h->tickets + kMaxTickets / 2;   // Gram launches of a handle follow one another
+    ProfScope ps(h, gram_kind(tp.prec), 4.0 * in.N * in.M + (in.w ? 4.0 * in.M : 0.0), tp.flops, s);
+    const cudaError_t e = launch_gram_cluster(cp, in.w, sqrt_w, tp.prec, tp.clusters, s);
+    if (e != cudaSuccess) return cuda_fail(h, e, "cluster Gram launch");
+    return PID_OK;
   }
   const int64_t plane = rup(static_cast<int64_t>(in.N) * tp.ldo * tp.elem_bytes, 1024);
   char* hi = static_cast<char*>(op);

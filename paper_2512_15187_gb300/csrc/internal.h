@@ -161,6 +161,24 @@ struct TiledParams {
   uint32_t* err;
 };
 
+// Gram of 256 < N <= 512 members in one pass, a cluster of R CTAs per cell chunk (gram_cluster.cu).
+struct ClusterGramParams {
+  const float* F;          // [N][ld] soft masks, or fields mapped by iso_mode
+  const float* sqrt_w;     // roots of the cell measures, zero up to a multiple of 128, or nullptr
+  float* gpart;            // [n_chunks][N][N] FP32 partial Grams (G_ij at j*N + i)
+  const float* op_scale;   // E4M3: [2N] per-member scales s_i, then 1/s_i (nullptr = 256)
+  unsigned int* flags;     // [clusters][R]: accumulators left for the next cluster
+  int64_t ld;
+  int32_t N, M, R;         // members, cells, 128-row blocks (3 or 4)
+  int32_t chunk_cells;     // multiple of 128
+  int32_t n_chunks;
+  int32_t stages;          // operand stages in the ring (gram_cluster_stages)
+  int32_t vec_ok;          // rows 16-byte aligned: 4-cell vector loads
+  int32_t iso_mode;
+  float iso_mu, iso_inv, iso_t;
+  uint32_t* err;
+};
+
 // Finalisation of one ensemble: fixed-order reduction of the chunk partials, then inclusion
 // fractions, depth and rank (finalize.cu; ensembles of more than 512 members: blocked.cu).
 enum FinKind : int32_t {
@@ -273,6 +291,10 @@ cudaError_t launch_member_scales(const ScaleBatchParams& p, cudaStream_t s);
 // reduction keys (maxima reduced by a streaming pass) or [N][segs] CTA maxima.
 constexpr size_t kScaleBytes = 8192;
 constexpr int kScaleMaxSlots = static_cast<int>(kScaleBytes / 4) - 2 * kGramTiledMaxN;
+cudaError_t launch_gram_cluster(const ClusterGramParams& p, const float* w, float* sqrt_w, int prec, int clusters,
+                                cudaStream_t s);
+cudaError_t gram_max_clusters(int R, int* clusters);
+int gram_cluster_stages(int R, int prec);
 // Row-block-tiled Gram (gram_tiled.cu).
 cudaError_t launch_gram_operands(const OperandParams& p, int prec, cudaStream_t s);
 cudaError_t launch_gram_tiled(const TiledParams& p, int prec, int grid, size_t smem, cudaStream_t s);
