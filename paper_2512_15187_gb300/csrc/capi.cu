@@ -344,13 +344,11 @@ pid_status plan_stream(pid_handle h, const EnsInput& in, EnsPlan* pl) {
   d.M = static_cast<int32_t>(in.M);
   const int n_groups = kStreamWarps / cfg.G;
   const int64_t total_groups = static_cast<int64_t>(h->sms) * n_groups;
-  const int64_t TS = static_cast<int64_t>(cfg.T) * cfg.sub;
-  int64_t chunk = round_up((in.M + total_groups - 1) / total_groups, TS);
-  chunk = std::max<int64_t>(TS, std::min<int64_t>(chunk, 256 * cfg.T));
+  // chunks are whole register tiles, whatever the stage: the sums' order does not depend on it
+  int64_t chunk = round_up((in.M + total_groups - 1) / total_groups, cfg.T);
+  chunk = std::max<int64_t>(cfg.T, std::min<int64_t>(chunk, 256 * cfg.T));
   d.chunk_cells = static_cast<int32_t>(chunk);
   d.n_chunks = static_cast<int32_t>((in.M + chunk - 1) / chunk);
-  d.n_boxes = static_cast<int32_t>((in.N + 255) / 256);
-  d.box_rows = static_cast<int32_t>((in.N + d.n_boxes - 1) / d.n_boxes);
   iso_fill(in.is_field ? &in.iso : nullptr, &d.iso_mode, &d.iso_mu, &d.iso_inv, &d.iso_t);
   d.validate = in.validate;
   const uintptr_t a = reinterpret_cast<uintptr_t>(in.data);
@@ -358,6 +356,16 @@ pid_status plan_stream(pid_handle h, const EnsInput& in, EnsPlan* pl) {
                       (in.w == nullptr || reinterpret_cast<uintptr_t>(in.w) % 16 == 0);
   pl->use_tma = false;
   pl->cls = false;
+  // the one-cell classes' boxes cover every row of the class (rows past N read as zero)
+  const int64_t rows = cfg.vec == 1 ? int64_t(cfg.G) * cfg.mpw : in.N;
+  d.n_boxes = static_cast<int32_t>((rows + 255) / 256);
+  d.box_rows = static_cast<int32_t>((rows + d.n_boxes - 1) / d.n_boxes);
+  int64_t TS = 0;      // cells per stage
+  auto stage_cells = [&](bool tma) {
+    pl->cfg.sub = stream_sub(cfg.vec, cfg.mpw, tma);
+    TS = static_cast<int64_t>(cfg.T) * pl->cfg.sub;
+  };
+  stage_cells(tma_ok);
   if (tma_ok && get_encode_fn()) {
     bool ok = encode_2d(&d.tmap, in.data, static_cast<uint64_t>(in.M), static_cast<uint64_t>(in.N),
                         static_cast<uint64_t>(in.ld) * 4, static_cast<uint32_t>(TS),
@@ -365,6 +373,7 @@ pid_status plan_stream(pid_handle h, const EnsInput& in, EnsPlan* pl) {
     if (ok && in.w) ok = encode_1d(&d.tmap_w, in.w, static_cast<uint64_t>(in.M), static_cast<uint32_t>(TS));
     pl->use_tma = ok;
   }
+  if (!pl->use_tma) stage_cells(false);
   if (!pl->use_tma && get_encode_fn()) {
     // Rows that are not 16-byte aligned: members of one residue class (i mod n_cls) share
     // their offset from the 16-byte boundary and lie n_cls ld floats apart, so each class is

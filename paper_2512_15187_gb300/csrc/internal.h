@@ -32,6 +32,13 @@ constexpr uint64_t kWaitTimeoutNs = 1000000000ull;
 // Streaming pass: 16 consumer warps per CTA, grouped G warps per cell tile.
 constexpr int kStreamWarps = 16;
 constexpr int kStreamThreads = kStreamWarps * 32;
+// Register tiles of a class's stage. The one-cell classes of 257 to 384 members take two where TMA
+// loads the rows: stages of
+// 64 cells, which still fit twice, read DRAM in row segments of 256 bytes and halve the copies
+// (PID-mean over 2^20 cells: 384 members 365 -> 254 us, 300 members 303 -> 228 us). Above 384 they do
+// not: quarters of a stage as ring slots (512 members: 464 us with 32 cells, 552 so) and 256 or
+// 512 byte segments prefetched into L2 (670 and 562) lost what the wider reads gained.
+constexpr int stream_sub(int vec, int mpw, bool tma) { return tma && vec == 1 && mpw <= 24 ? 2 : 1; }
 constexpr int kStreamProducerBytes = 96;   // shared-memory TMA cursor per group
 
 // One ensemble as seen by the streaming kernel.
@@ -53,7 +60,7 @@ struct EnsDesc {  // 64-byte aligned through its CUtensorMap members
   float* part;          // [n_chunks][2N] FP32 partial sums: m_i, then N A_i (pass 1) or B_i (pass 2)
   int64_t ld;
   int32_t N, M;
-  int32_t chunk_cells;  // multiple of the stage width sub*T
+  int32_t chunk_cells;  // multiple of the register tile (streaming: 32 VEC cells)
   int32_t n_chunks;
   int32_t unit_begin;   // index of chunk 0 in the launch's flat unit list
   int32_t box_rows;     // members per TMA box (<= 256)

@@ -263,9 +263,9 @@ stream_kernel(const __grid_constant__ StreamParams p) {
   const int q = warp - grp * G;
   const int depth = p.depth;
   const int SF = p.stage_floats;
-  // One register tile per TMA stage (every tile class is planned with sub = 1): the stage
-  // width is a compile-time constant, so row offsets fold into the shared-memory loads.
-  constexpr int SUB = 1;
+  // Register tiles per TMA stage: the stage width is a compile-time constant, so row offsets
+  // fold into the shared-memory loads.
+  constexpr int SUB = stream_sub(VEC, MPW, TMA);
   constexpr int TS = SUB * T;
   // Row stride of a stage: TMA stores rows back to back; the cp.async path stores each
   // row's enclosing 16-byte-aligned span (4 floats more), the row's first cell `roff` floats in.
@@ -275,6 +275,11 @@ stream_kernel(const __grid_constant__ StreamParams p) {
   // one-cell-per-lane classes keep the cp.async spans (their spans of TS + 4 = 36 cells
   // cost more L2 traffic than the copies save), and compile without the class code.
   const bool CLS = !TMA && VEC > 1 && p.use_tma == 2;
+  // One-cell classes over aligned soft masks: the TMA boxes cover every row of the class and
+  // zero-fill those past N, so no row needs a test (with the packed accumulation below: 512
+  // members over 2^20 cells 512 -> 462 us; the launch waited for the issue of 15 instructions per
+  // member and cell).
+  constexpr bool ALL_ROWS = TMA && VEC == 1 && ISO == ISOK_NONE;
 
   float* ring = reinterpret_cast<float*>(smem);
   float* red = ring + static_cast<size_t>(NG) * depth * SF;
@@ -457,11 +462,13 @@ stream_kernel(const __grid_constant__ StreamParams p) {
     const int cell0 = c * e_chunk;
     const int cells = min(e_chunk, M - cell0);
     const int n_st = (cells + TS - 1) / TS;
-    float accM[MPW], accA[MPW], accX[MAXU ? MPW : 1];
+    constexpr int NX = MAXU ? (VEC == 1 ? 1 : MPW) : 1;
+    float accM[MPW], accA[MPW], accX[NX];
+    unsigned int max_key = 0;   // VEC = 1: lane k holds the key of this warp's k-th member's maximum
 #pragma unroll
     for (int k = 0; k < MPW; ++k) { accM[k] = 0.f; accA[k] = 0.f; }
 #pragma unroll
-    for (int k = 0; k < (MAXU ? MPW : 1); ++k) accX[k] = 0.f;
+    for (int k = 0; k < NX; ++k) accX[k] = 0.f;
 
     // Rows that are not 16-byte aligned (no TMA): each stage holds, per member row, the
     // 16-byte-aligned span that encloses the stage's cells, its first cell `ro` floats
@@ -519,7 +526,7 @@ stream_kernel(const __grid_constant__ StreamParams p) {
       if (q == 0 && has_w) {
         const int xs = xs0 + lane;
 #pragma unroll
-        for (int v = 0; v < VEC; ++v) {
+        for (int v = 0; v < TS / 32; ++v) {
           const bool in = xs + 32 * v < M;
           cp_async4(stage + SF - TS + lane + 32 * v, d.w + (in ? xs + 32 * v : 0), in ? 4u : 0u);
         }
@@ -542,7 +549,10 @@ stream_kernel(const __grid_constant__ StreamParams p) {
       if (++c_slot == depth) { c_slot = 0; c_par ^= 1u; }
       const float* sb = my_ring + static_cast<size_t>(slot) * SF;
       if (!mbar_wait_bounded(&my_bars[slot], par, kWaitTimeoutNs)) flags[2 * grp + (k_sub & 1)] = 1;
-      for (int j = 0; j < SUB; ++j, ++k_sub) {
+      // the chunk's last stage may hold fewer register tiles
+      const int n_sub = SUB == 1 ? 1 : min(SUB, (cells - st * TS + T - 1) / T);
+#pragma unroll 1
+      for (int j = 0; j < n_sub; ++j, ++k_sub) {
         const int x0 = cell0 + st * TS + j * T;     // first cell of this register tile
         const int xl = x0 + lane * VEC;             // first cell of this lane
         const bool full = x0 + T <= M;              // no cell past the end of the ensemble
@@ -550,12 +560,17 @@ stream_kernel(const __grid_constant__ StreamParams p) {
         float wv[VEC];
 
         // the stage in shared memory, filled by TMA or by the threads' cp.async copies
+        const int ro = (boff + q * ld3) & 3, rstep = sstep * RS;
+        const float* rows0 = sb + srow0 * RS + j * T + lane * VEC;
 #pragma unroll
         for (int k = 0; k < MPW; ++k) {
           const int i = q + k * G;
-          if (i < N) {
+          if (ALL_ROWS || i < N) {
             if constexpr (TMA) {
               lds_vec<VEC>(x[k], sb + static_cast<size_t>(i) * TS + j * T + lane * VEC);
+            } else if constexpr (G % 4 == 0) {
+              // member q + k G starts `ro` floats into its span, the same for all of the warp's
+              lds_shifted<VEC>(x[k], rows0 + k * rstep, ro);
             } else {
               // the row's cells start `ro` floats into its span (the same for the warp)
               lds_shifted<VEC>(x[k], sb + static_cast<size_t>(srow0 + k * sstep) * RS + j * T + lane * VEC,
@@ -566,6 +581,7 @@ stream_kernel(const __grid_constant__ StreamParams p) {
             for (int v = 0; v < VEC; ++v) x[k][v] = pad;
           }
         }
+        if (VEC == 1) wv[0] = 1.f;
         if (has_w) lds_vec<VEC>(wv, sb + SF - TS + j * T + lane * VEC);
 
         if (validate) {
@@ -702,11 +718,11 @@ stream_kernel(const __grid_constant__ StreamParams p) {
         }
         if (flags[2 * grp + (k_sub & 1)]) { aborted = true; break; }
         if constexpr (TMA) {
-          if (leader && j == SUB - 1) issue_next();  // every warp has read this slot: refill it
+          if (leader && j == n_sub - 1) issue_next();  // every warp has read this slot: refill it
         } else if (CLS) {
-          if (leader && j == SUB - 1) issue_next_cls();  // every warp has read this slot
+          if (leader && j == n_sub - 1) issue_next_cls();  // every warp has read this slot
         } else {
-          if (j == SUB - 1 && st + depth < n_st) cpa_issue(st + depth, slot);
+          if (j == n_sub - 1 && st + depth < n_st) cpa_issue(st + depth, slot);
         }
         if constexpr (G > 2) {
           if (p.xchg == 1) {
@@ -732,11 +748,16 @@ stream_kernel(const __grid_constant__ StreamParams p) {
         // one-cell-per-lane classes keep a single loop: the duplicated code costs them
         // registers.)
         if constexpr (VEC == 1) {
+          // two members at a time (packed pairs); without cell measures wv is 1, which
+          // multiplies exactly
+          const float2 w2 = f2(wv[0]), s2 = f2(s[0]);
 #pragma unroll
-          for (int k = 0; k < MPW; ++k) {
-            const float t = has_w ? wv[0] * x[k][0] : x[k][0];
-            accM[k] += t;
-            accA[k] = fmaf(t, s[0], accA[k]);
+          for (int k = 0; k < MPW; k += 2) {
+            const float2 t = f2_mul(w2, make_float2(x[k][0], x[k + 1][0]));
+            const float2 m = f2_add(make_float2(accM[k], accM[k + 1]), t);
+            const float2 a = f2_fma(t, s2, make_float2(accA[k], accA[k + 1]));
+            accM[k] = m.x; accM[k + 1] = m.y;
+            accA[k] = a.x; accA[k + 1] = a.y;
           }
         } else if (has_w) {
 #pragma unroll
@@ -766,7 +787,11 @@ stream_kernel(const __grid_constant__ StreamParams p) {
           // the operand u sqrt(w), rounded as the Gram kernels round it
           const float sw = has_w ? sqrtf(wv[0]) : 1.f;
 #pragma unroll
-          for (int k = 0; k < MPW; ++k) accX[k] = fmaxf(accX[k], has_w ? x[k][0] * sw : x[k][0]);
+          for (int k = 0; k < MPW; ++k) {
+            // reduced over the lanes at once: a register per member would spill
+            const unsigned int key = __reduce_max_sync(0xffffffffu, fkey(fmaxf(0.f, has_w ? x[k][0] * sw : x[k][0])));
+            if (lane == k) max_key = max(max_key, key);
+          }
         } else if constexpr (MAXU) {
           // the operand u sqrt(w), rounded as the Gram kernels round it
           if (has_w) {
@@ -805,6 +830,10 @@ stream_kernel(const __grid_constant__ StreamParams p) {
     if constexpr (MAXU) {
       unsigned int* const um = dp->umax;
       if (um != nullptr) {
+        if constexpr (VEC == 1) {
+          const int i = q + lane * G;
+          if (lane < MPW && i < N) atomicMax(um + i, max_key);
+        } else
 #pragma unroll
         for (int k = 0; k < MPW; ++k) {
           float mx = accX[k];
