@@ -184,7 +184,7 @@ __device__ __forceinline__ float iso_map(float f, float mu, float inv, float t, 
 struct StreamProducer {
   const EnsDesc* pd;   // descriptor of the ensemble being loaded
   long n_issued;       // stages issued so far
-  int iu, u_end;       // unit being loaded, end of the group's run
+  int iu, left;        // unit being loaded, units left (with it)
   int ist, in_st;      // stage within the unit, stages of the unit
   int icell0, slot;    // first cell of the unit, ring slot of the next stage
   int e_begin, e_end, chunk, M, boxes, rows, has_w;
@@ -317,10 +317,14 @@ stream_kernel(const __grid_constant__ StreamParams p) {
   const int u_begin = unit_at_work(p, p.total_work * gid / total_groups);
   const int u_end = unit_at_work(p, p.total_work * (gid + 1) / total_groups);
 
+  // The second pass takes a group's units in reverse: the data (or the stored masks) that the first
+  // pass touched last are still in L2. Units do not depend on one another, so the results do not change.
+  constexpr bool BACK = COEF;
+
   // ---- producer cursor (leader lane of the group only, in shared memory) ----
   StreamProducer& P = prod[grp];
   auto set_unit = [&](int u) {
-    if (u >= P.e_end) {
+    if (u >= P.e_end || u < P.e_begin) {
       const EnsDesc* pd = &stream_desc(p, stream_find_ens(p, u));
       P.pd = pd;
       P.e_begin = pd->unit_begin;
@@ -336,7 +340,7 @@ stream_kernel(const __grid_constant__ StreamParams p) {
     P.in_st = (min(P.chunk, P.M - P.icell0) + TS - 1) / TS;
   };
   auto issue_next = [&]() {
-    if (P.iu >= P.u_end) return;
+    if (P.left <= 0) return;
     const int slot = P.slot;
     P.slot = slot + 1 == depth ? 0 : slot + 1;
     float* dst = my_ring + static_cast<size_t>(slot) * SF;
@@ -352,14 +356,14 @@ stream_kernel(const __grid_constant__ StreamParams p) {
     ++P.n_issued;
     if (++P.ist == P.in_st) {
       P.ist = 0;
-      if (++P.iu < P.u_end) set_unit(P.iu);
+      if (--P.left > 0) set_unit(P.iu += BACK ? -1 : 1);
     }
   };
   // Unaligned rows through the class maps: class c's boxes fill the stage rows from
   // c n_boxes box_rows on, each row the 16-byte-aligned span of TS + 4 cells around the
   // stage's cells (its first cell (data + i ld) mod 16 bytes in); cells past M read as 0.
   auto issue_next_cls = [&]() {
-    if (P.iu >= P.u_end) return;
+    if (P.left <= 0) return;
     const int slot = P.slot;
     P.slot = slot + 1 == depth ? 0 : slot + 1;
     float* dst = my_ring + static_cast<size_t>(slot) * SF;
@@ -379,14 +383,14 @@ stream_kernel(const __grid_constant__ StreamParams p) {
     ++P.n_issued;
     if (++P.ist == P.in_st) {
       P.ist = 0;
-      if (++P.iu < P.u_end) set_unit(P.iu);
+      if (--P.left > 0) set_unit(P.iu += BACK ? -1 : 1);
     }
   };
   if (leader) {
     P.pd = nullptr;
     P.n_issued = 0;
-    P.iu = u_begin;
-    P.u_end = u_end;
+    P.iu = BACK ? u_end - 1 : u_begin;
+    P.left = u_end - u_begin;
     P.ist = 0;
     P.in_st = 0;
     P.icell0 = 0;
@@ -394,10 +398,10 @@ stream_kernel(const __grid_constant__ StreamParams p) {
     P.e_begin = 0;
     P.e_end = 0;
     if (TMA) {
-      if (P.iu < P.u_end) set_unit(P.iu);
+      if (P.left > 0) set_unit(P.iu);
       for (int s = 0; s < depth; ++s) issue_next();
     } else if (CLS) {
-      if (P.iu < P.u_end) set_unit(P.iu);
+      if (P.left > 0) set_unit(P.iu);
       for (int s = 0; s < depth; ++s) issue_next_cls();
     }
   }
@@ -422,8 +426,8 @@ stream_kernel(const __grid_constant__ StreamParams p) {
   // spans keep member order (row q + k G); with class maps the member q + k G sits in the
   // slot of class q mod n_cls, at row (q + k G) / n_cls (G is a multiple of n_cls).
   int srow0 = q, sstep = G;
-  for (int u = u_begin; u < u_end && !aborted; ++u) {
-    if (u >= e_end) {
+  for (int n = u_end - u_begin, u = BACK ? u_end - 1 : u_begin; n > 0 && !aborted; --n, u += BACK ? -1 : 1) {
+    if (u >= e_end || u < e_begin) {
       dp = &stream_desc(p, stream_find_ens(p, u));
       if constexpr (!TMA) {
         if (CLS) {
