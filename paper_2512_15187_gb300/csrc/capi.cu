@@ -499,6 +499,7 @@ pid_status stream_launch(pid_handle h, StreamParams sp, const StreamCfg& cfg, bo
     std::pair<int, int> pick{sp.xchg, dmax};
     for (auto c : cand) {
       StreamParams t = sp;
+      t.pdl = 0;
       t.xchg = c.first;
       t.depth = c.second;
       const size_t sm = stream_smem_bytes(cfg.vec, cfg.G, c.second, sp.stage_floats);
@@ -566,7 +567,8 @@ pid_status ensure_workspace(pid_handle h, size_t bytes, cudaStream_t s) {
 // Launch sequences for one ensemble (single calls)
 // ---------------------------------------------------------------------------------------
 
-static pid_status launch_stream_one(pid_handle h, EnsPlan& pl, const float* coef, cudaStream_t s) {
+static pid_status launch_stream_one(pid_handle h, EnsPlan& pl, const float* coef, cudaStream_t s,
+                                    bool behind_fin = false) {
   StreamParams sp;
   std::memset(&sp, 0, sizeof(sp));
   sp.one = pl.desc;
@@ -584,6 +586,7 @@ static pid_status launch_stream_one(pid_handle h, EnsPlan& pl, const float* coef
   sp.stage_floats = pl.stage_floats;
   if (coef) sp.one.umax = nullptr;
   sp.maxu = sp.one.umax != nullptr ? 1 : 0;
+  sp.pdl = behind_fin ? 1 : 0;
   const int n_groups = kStreamWarps / pl.cfg.G;
   int grid = std::min<int>(h->sms, (sp.total_units + n_groups - 1) / n_groups);
   grid = std::max(grid, 1);
@@ -758,7 +761,9 @@ pid_status run_single(pid_handle h, const EnsInput& in, const EnsOutputs& out, c
   f1.depth = nullptr; f1.in_in = nullptr; f1.in_out = nullptr; f1.rank = nullptr;
   st = launch_fin_one(h, f1, s);
   if (st != PID_OK) return st;
-  st = launch_stream_one(h, pl, coef, s);
+  // Loads of the second pass start while the first one's finalisation runs (it reads the data, which
+  // nobody here writes, before it waits).
+  st = launch_stream_one(h, pl, coef, s, true);
   if (st != PID_OK) return st;
   FinDesc f2 = fd;
   f2.kind = FIN_LIN2;

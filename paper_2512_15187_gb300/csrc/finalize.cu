@@ -167,6 +167,7 @@ finalize_kernel(const __grid_constant__ FinParams p) {
   __shared__ FinShared sh;
   cluster_arrive();                      // every CTA has started before its memory is written
   grid_dependency_wait();
+  grid_launch_dependents();              // a second pass may start loading (it waits for this grid's end)
   const FinDesc& d = fin_desc(p, blockIdx.y);
   const int rank = static_cast<int>(blockIdx.x);
   const FinSpan sp = fin_span(d.N, rank);

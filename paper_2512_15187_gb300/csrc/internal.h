@@ -97,7 +97,7 @@ struct StreamParams {
   int32_t xchg;            // column-sum exchange: 0 direct, 1 reduce-scatter (G > 2)
   uint32_t* err;           // device error word
   int32_t maxu;            // some descriptor has umax: the instantiation that tracks maxima
-  int32_t pad;
+  int32_t pdl;             // coefficient pass behind the finalisation that writes them: may start early
 };
 
 // Tensor-core Gram pass: 16 warps convert tiles (the streaming arithmetic plus operand

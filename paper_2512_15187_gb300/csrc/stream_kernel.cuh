@@ -406,6 +406,10 @@ stream_kernel(const __grid_constant__ StreamParams p) {
     }
   }
 
+  // A second pass launched behind the first one's finalisation has filled its ring by now; the
+  // coefficients, and the partials that the finalisation reads, wait for its end.
+  if constexpr (COEF) grid_dependency_wait();
+
   // ---- consumers: every warp of the group ----
   long k_cons = 0;
   int c_slot = 0;
@@ -866,6 +870,19 @@ stream_kernel(const __grid_constant__ StreamParams p) {
 
 template <int VEC, int MPW, int G, int ISO, bool COEF, bool TMA, bool MAXU = false>
 cudaError_t launch_stream_inst(const StreamParams& p, int grid, size_t smem, cudaStream_t s) {
+  if (COEF && p.pdl) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(grid));
+    cfg.blockDim = dim3(kStreamThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, stream_kernel<VEC, MPW, G, ISO, COEF, TMA, MAXU>, p);
+  }
   stream_kernel<VEC, MPW, G, ISO, COEF, TMA, MAXU><<<grid, kStreamThreads, smem, s>>>(p);
   return cudaGetLastError();
 }
