@@ -290,9 +290,11 @@ def _ptr(t):
 
 
 def _stream(stream):
+    if stream is not None:
+        return stream.cuda_stream
+    # the current stream's handle without building a torch.cuda.Stream (2.9 us of a small call's 27)
     import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return c_void_p(s.cuda_stream)
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _check_matrix(x, name):
