@@ -35,6 +35,13 @@ __device__ __forceinline__ const FinDesc& fin_desc(const FinParams& p, int e) {
   return p.descs ? p.descs[e] : p.one;
 }
 
+// The barrier of an ensemble's C CTAs.
+template <int C>
+__device__ __forceinline__ void fin_sync() {
+  if constexpr (C == 1) __syncthreads();
+  else cluster_sync_all();
+}
+
 // State shared by the members of one CTA.
 struct FinShared {
   float2 acc[kFinThreads];              // partial column sums
@@ -47,9 +54,10 @@ struct FinShared {
 struct FinSpan {
   int N, m0, nm, cp;
 };
+template <int C>
 __device__ __forceinline__ FinSpan fin_span(int N, int rank) {
   FinSpan s;
-  const int per = (N + kFinCtas - 1) / kFinCtas;
+  const int per = (N + C - 1) / C;
   s.N = N;
   s.m0 = min(N, rank * per);
   s.nm = min(N, s.m0 + per) - s.m0;
@@ -122,22 +130,26 @@ __device__ void fin_reduce(FinShared& sh, const float* part, int rows, const Fin
 
 // The sum of x over all members: every CTA sums its own (xor tree over 64 slots), pushes the
 // result to all CTAs; the cluster barrier that must follow makes csum readable.
+template <int C>
 __device__ __forceinline__ void fin_push_sum(FinShared& sh, double x_lo, double x_hi, int rank) {
   if (threadIdx.x < 32) {
     const double s = warp_sum(x_lo + x_hi);
-    if (threadIdx.x < kFinCtas) st_cluster(cluster_addr(&sh.csum[rank], threadIdx.x), s);
+    if (threadIdx.x < C) st_cluster(cluster_addr(&sh.csum[rank], threadIdx.x), s);
   }
 }
+template <int C>
 __device__ __forceinline__ double fin_total(const FinShared& sh) {
-  static_assert(kFinCtas == 8, "pairwise sum of eight");
+  if constexpr (C == 1) return sh.csum[0];
+  static_assert(C == 1 || C == 8, "pairwise sum of eight");
   return ((sh.csum[0] + sh.csum[1]) + (sh.csum[2] + sh.csum[3])) +
          ((sh.csum[4] + sh.csum[5]) + (sh.csum[6] + sh.csum[7]));
 }
 
+template <int C>
 __device__ __forceinline__ void fin_push_key(FinShared& sh, int i, double depth) {
   const unsigned long long k = order_key(depth);
 #pragma unroll
-  for (int r = 0; r < kFinCtas; ++r) st_cluster(cluster_addr(&sh.key[i], r), k);
+  for (int r = 0; r < C; ++r) st_cluster(cluster_addr(&sh.key[i], r), k);
 }
 
 // Ranks of this CTA's members: one warp per member counts the members that are deeper, or as
@@ -170,7 +182,7 @@ finalize_kernel(const __grid_constant__ FinParams p) {
   grid_launch_dependents();              // a second pass may start loading (it waits for this grid's end)
   const FinDesc& d = fin_desc(p, blockIdx.y);
   const int rank = static_cast<int>(blockIdx.x);
-  const FinSpan sp = fin_span(d.N, rank);
+  const FinSpan sp = fin_span<kFinCtas>(d.N, rank);
   const int N = sp.N, t = threadIdx.x;
   const int kind = d.kind;
   const bool wm = kind == FIN_WMEAN, second = kind == FIN_LIN2;
@@ -192,9 +204,9 @@ finalize_kernel(const __grid_constant__ FinParams p) {
       if (t + 32 < sp.nm)
         hi = wm ? sh.tot[t + 32] * static_cast<double>(__ldcg(d.coef + sp.m0 + t + 32)) : sh.tot[t + 32];
     }
-    fin_push_sum(sh, lo, hi, rank);
+    fin_push_sum<kFinCtas>(sh, lo, hi, rank);
     cluster_sync_all();
-    if (mine) msum = fin_total(sh);
+    if (mine) msum = fin_total<kFinCtas>(sh);
   }
   double depth = 0.0;
   if (mine) {
@@ -220,7 +232,7 @@ finalize_kernel(const __grid_constant__ FinParams p) {
     }
   }
   if (kind != FIN_LIN1 && d.rank != nullptr) {
-    if (mine) fin_push_key(sh, i, depth);
+    if (mine) fin_push_key<kFinCtas>(sh, i, depth);
     cluster_sync_all();
     fin_ranks(sh, sp, d.rank);
   }
@@ -316,9 +328,12 @@ __global__ void __launch_bounds__(kGramSumThreads) gram_sum_kernel(const __grid_
 // Each CTA keeps its members' rows of the symmetrised Gram in shared memory (64 x 512 floats at
 // N = 512; rows padded to an odd stride so that the transposed half writes without bank
 // conflicts) and its warps dot them with the scales, which every sweep pushes to all CTAs.
+// Small ensembles with few chunks take one CTA (fin_gram_single): a sweep then costs a CTA barrier
+// instead of a cluster's (20 x 128^2 BF16 with P: 35.0 -> 30.8 us a call).
 // 512 x 2^20 split BF16 with P: the whole call 2806 -> 2411 us against one CTA that did all of
 // this (437 us); the plume step's three items 1076 -> 996 us (131 us).
-__global__ void __cluster_dims__(kFinCtas, 1, 1) __launch_bounds__(kFinThreads, 1)
+template <int CTAS>
+__global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(kFinThreads, 1)
 finalize_gram_kernel(const __grid_constant__ FinParams p) {
   extern __shared__ float fin_c0[];                     // [nm][N | 1]
   __shared__ FinShared sh;
@@ -326,12 +341,12 @@ finalize_gram_kernel(const __grid_constant__ FinParams p) {
   __shared__ float starget[kFinMaxRows], sraw[kFinMaxRows];
   __shared__ int smoved[2][kFinCtas];
   __shared__ double serr[kFinCtas];
-  cluster_arrive();
+  if constexpr (CTAS > 1) cluster_arrive();
   grid_dependency_wait();
   grid_launch_dependents();
   const FinDesc& d = fin_desc(p, blockIdx.y);
   const int rank = static_cast<int>(blockIdx.x);
-  const FinSpan sp = fin_span(d.N, rank);
+  const FinSpan sp = fin_span<CTAS>(d.N, rank);
   const int N = sp.N, t = threadIdx.x, warp = t >> 5, lane = t & 31;
   const int stride = N | 1;
   float* const G = fin_gram(d);
@@ -346,16 +361,16 @@ finalize_gram_kernel(const __grid_constant__ FinParams p) {
   const int i = sp.m0 + t;
   const bool mine = t < sp.nm;
   const double m = mine ? sh.tot[t] : 0.0, A = mine ? sh.tot[kFinMaxRows + t] : 0.0;   // m_i, N A_i
-  cluster_wait();
+  if constexpr (CTAS > 1) cluster_wait();
   {
     double lo = 0.0, hi = 0.0;
     if (t < 32) {
       if (t < sp.nm) lo = sh.tot[t];
       if (t + 32 < sp.nm) hi = sh.tot[t + 32];
     }
-    fin_push_sum(sh, lo, hi, rank);
+    fin_push_sum<CTAS>(sh, lo, hi, rank);
   }
-  cluster_sync_all();    // the other CTAs' shares of the mass; their rows of G (inline sums)
+  fin_sync<CTAS>();    // the other CTAs' shares of the mass; their rows of G (inline sums)
 
   // Row r of the stored array is G'_{., r}, which equals row r of G' up to the rounding of the
   // tensor-core sums: its raw sum, and one half of C0.
@@ -403,7 +418,7 @@ finalize_gram_kernel(const __grid_constant__ FinParams p) {
   }
   double in_in = 0.0, err = 0.0;
   if (mine) {
-    const double msum = fin_total(sh);
+    const double msum = fin_total<CTAS>(sh);
     const double nm_i = m * N;
     in_in = m > 0.0 ? A / nm_i : 0.0;
     if (d.mean_depth) d.mean_depth[i] = fmin(in_in, msum > 0.0 ? A / msum : 0.0);
@@ -413,9 +428,9 @@ finalize_gram_kernel(const __grid_constant__ FinParams p) {
     starget[t] = static_cast<float>(A);                 // row-sum target N A_i
     const float s0 = (A > 0.0 && raw > 0.0) ? 1.0f : 0.0f;
 #pragma unroll
-    for (int r = 0; r < kFinCtas; ++r) st_cluster(cluster_addr(&sd[0][i], r), s0);
+    for (int r = 0; r < CTAS; ++r) st_cluster(cluster_addr(&sd[0][i], r), s0);
   }
-  cluster_sync_all();
+  fin_sync<CTAS>();
   // Symmetric Sinkhorn: d_r <- sqrt(d_r N A_r / sum_j C0_rj d_j), until no scale moves by more
   // than 2^-22 relative (at most 24 sweeps).
   int cur = 0;
@@ -430,15 +445,15 @@ finalize_gram_kernel(const __grid_constant__ FinParams p) {
         const float so = sd[cur][sp.m0 + r];
         const float sn = (so > 0.f && acc[k] > 0.f) ? sqrtf(so * starget[r] / acc[k]) : 0.f;
         moved = moved || fabsf(sn - so) > 2.4e-7f * so;
-        if (lane < kFinCtas) st_cluster(cluster_addr(&sd[cur ^ 1][sp.m0 + r], lane), sn);
+        if (lane < CTAS) st_cluster(cluster_addr(&sd[cur ^ 1][sp.m0 + r], lane), sn);
       }
     }
     const int any = __syncthreads_or(moved);
-    if (t < kFinCtas) st_cluster(cluster_addr(&smoved[cur][rank], t), any);
-    cluster_sync_all();
+    if (t < CTAS) st_cluster(cluster_addr(&smoved[cur][rank], t), any);
+    fin_sync<CTAS>();
     int more = 0;
 #pragma unroll
-    for (int r = 0; r < kFinCtas; ++r) more |= smoved[cur][r];
+    for (int r = 0; r < CTAS; ++r) more |= smoved[cur][r];
     cur ^= 1;
     if (!more) break;
   }
@@ -447,10 +462,10 @@ finalize_gram_kernel(const __grid_constant__ FinParams p) {
   if (mine) {
     const float dm = m > 0.0 ? static_cast<float>(static_cast<double>(sd[cur][i]) / m) : 0.f;
 #pragma unroll
-    for (int r = 0; r < kFinCtas; ++r) st_cluster(cluster_addr(&sdm[i], r), dm);
+    for (int r = 0; r < CTAS; ++r) st_cluster(cluster_addr(&sdm[i], r), dm);
     if (d.P) inv_m = m > 0.0 ? 1.0 / m : 0.0;
   }
-  cluster_sync_all();
+  fin_sync<CTAS>();
   {
     float acc[kFinRowsPerWarp];
     rows_dot(fin_c0, stride, sp.nm, sdm, N, acc);
@@ -468,7 +483,7 @@ finalize_gram_kernel(const __grid_constant__ FinParams p) {
     if (d.depth) d.depth[i] = depth;
     if (d.in_in) d.in_in[i] = in_in;
     if (d.in_out) d.in_out[i] = in_out;
-    if (d.rank) fin_push_key(sh, i, depth);
+    if (d.rank) fin_push_key<CTAS>(sh, i, depth);
     if (d.P) sh.tot[t] = inv_m;          // 1 / m_i: m is in the owner's registers by now
   }
   if (d.err_est) {
@@ -484,11 +499,11 @@ finalize_gram_kernel(const __grid_constant__ FinParams p) {
       st_cluster(cluster_addr(&serr[rank], 0), e);
     }
   }
-  cluster_sync_all();
+  fin_sync<CTAS>();
   if (d.err_est && rank == 0 && t == 0) {
     double e = serr[0];
 #pragma unroll
-    for (int r = 1; r < kFinCtas; ++r) e = fmax(e, serr[r]);
+    for (int r = 1; r < CTAS; ++r) e = fmax(e, serr[r]);
     d.err_est[0] = e;
   }
   if (d.rank) fin_ranks(sh, sp, d.rank);
@@ -525,7 +540,7 @@ __global__ void __launch_bounds__(256) gram_matrix_kernel(const __grid_constant_
 }
 
 cudaError_t finalize_kernels_init() {
-  return cudaFuncSetAttribute(finalize_gram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  return cudaFuncSetAttribute(finalize_gram_kernel<kFinCtas>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               kFinMaxRows * (kFinMaxN | 1) * static_cast<int>(sizeof(float)));
 }
 
@@ -561,8 +576,14 @@ cudaError_t launch_finalize(const FinParams& p, const FinLaunch& l, cudaStream_t
     if (e != cudaSuccess) return e;
     pdl = true;
   }
+  if (l.single) {
+    const size_t smem = static_cast<size_t>(l.max_n) * (l.max_n | 1) * sizeof(float);
+    e = fin_launch(finalize_gram_kernel<1>, dim3(1, grid.y), kFinThreads, smem, pdl, p, s);
+    if (e != cudaSuccess || !l.matrix) return e;
+    return fin_launch(gram_matrix_kernel, dim3((NN + 1023) / 1024, grid.y), 256, 0, true, p, s);
+  }
   const size_t rows = (static_cast<size_t>(l.max_n) + kFinCtas - 1) / kFinCtas;
-  e = fin_launch(finalize_gram_kernel, grid, kFinThreads, rows * (l.max_n | 1) * sizeof(float), pdl, p, s);
+  e = fin_launch(finalize_gram_kernel<kFinCtas>, grid, kFinThreads, rows * (l.max_n | 1) * sizeof(float), pdl, p, s);
   if (e != cudaSuccess || !l.matrix) return e;
   return fin_launch(gram_matrix_kernel, dim3((NN + 1023) / 1024, grid.y), 256, 0, true, p, s);
 }

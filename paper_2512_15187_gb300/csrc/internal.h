@@ -231,6 +231,7 @@ struct FinLaunch {
   bool sum_gram = false;   // some ensemble's Gram partials are summed by a launch of their own
   bool matrix = false;     // some ensemble wants P and its rows by a launch of their own
   bool pdl = false;        // the kernel before it in the stream is its producer
+  bool single = true;      // FIN_GRAM: every ensemble takes one CTA (fin_gram_single)
 };
 
 struct IsoParams {
@@ -246,6 +247,12 @@ struct IsoParams {
 // less); above this many bytes a launch over the whole GPU sums them first. 8 CTAs read about
 // 1 TB/s, so 2 MB cost them what the extra launch does.
 inline bool fin_gram_inline(int64_t N, int64_t n_gchunks) { return n_gchunks * N * N * 4 <= (int64_t(2) << 20); }
+// Ensembles that one CTA finalises: few members, and chunk sums small enough for one SM. The
+// finalisation with one CTA against a cluster of 8: 8 x 4096 16.9 and 22.6 us, 20 x 16 384 18.9 and
+// 22.5, 32 x 4096 20.1 and 22.6, but 64 x 4096 28.4 and 24.1.
+inline bool fin_gram_single(int64_t N, int64_t n_gchunks) {
+  return N <= 32 && n_gchunks * N * N * 4 <= (int64_t(128) << 10);
+}
 // Up to this many members the finalisation writes P itself; above, a launch over the whole
 // GPU does (N^2 FP64 products, at 2 per clock and SM).
 constexpr int kFinInlineMatrixN = 96;
