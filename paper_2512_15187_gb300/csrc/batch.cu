@@ -6,7 +6,7 @@
 // (ensemble, chunk) units; one finalisation launch then serves every ensemble. The exact
 // full PID adds a second streaming launch per class and a second finalisation. Full PID on
 // tensor cores runs one Gram launch per class instead of the first streaming pass; above 256
-// members the Gram is row-block-tiled (operands staged in HBM, one launch pair per ensemble)
+// members the Gram is row-block-tiled (clusters in one pass, or operands staged in HBM)
 // and the ensemble's exact PID-mean sums come from the first streaming pass of its class.
 // Items over the same data share first passes: a Gram item of soft masks takes the (m, A)
 // of a PID-mean or exact item's pass, and a PID-mean item those of an exact item's pass.

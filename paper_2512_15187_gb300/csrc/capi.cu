@@ -620,8 +620,9 @@ pid_status launch_member_coef_one(pid_handle h, const double* r, int64_t N, floa
 }
 
 // Full PID on the tensor cores for 256 < N <= 512: the streaming pass gives the exact
-// PID-mean sums (m_i, N A_i) that calibrate the Gram, the operand rows are staged in HBM,
-// the tiled kernel forms the chunk partial Grams, and the finalisation does the rest.
+// PID-mean sums (m_i, N A_i) that calibrate the Gram, the chunk partial Grams come from clusters in
+// one pass over the data or, for short ensembles, from operand rows staged in HBM and the tiled
+// kernel, and the finalisation does the rest.
 static pid_status run_gram_tiled(pid_handle h, const EnsInput& in, EnsPlan& pl,
                                  const EnsOutputs& out, cudaStream_t s) {
   TiledPlan tp;

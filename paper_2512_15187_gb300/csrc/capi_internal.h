@@ -137,8 +137,8 @@ struct GramPlan {
   double bytes = 0, flops = 0;
 };
 
-// Row-block-tiled Gram for 256 < N <= 512 (gram.cu, kernels in gram_tiled.cu): the
-// operand rows are staged in HBM and each CTA computes one tile of one cell chunk.
+// Gram of 256 < N <= 512 members (gram.cu): clusters in one pass over the data (gram_cluster.cu), or,
+// with few chunks, operand rows staged in HBM and a tile of a chunk per CTA (gram_tiled.cu).
 struct TiledPlan {
   int prec = 0;            // PID_BF16, PID_SPLIT_BF16 or PID_FP8
   int R = 0;               // 128-row blocks
@@ -153,7 +153,7 @@ struct TiledPlan {
   int n_gchunks = 0;
   int stages = 2;
   size_t smem = 0;
-  size_t op_bytes = 0;     // operand planes
+  size_t op_bytes = 0;     // operand planes, or (clusters) the roots of the cell measures
   size_t gpart_bytes = 0;  // [n_gchunks][N][N] float32
   double op_rw_bytes = 0, gemm_bytes = 0, flops = 0;
 };
