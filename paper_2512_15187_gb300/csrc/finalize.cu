@@ -2,11 +2,14 @@
 // fractions, depths and ranks of Eq. 10 / Eq. 16, and the calibration of the tensor-core
 // Gram.
 //
-// One cluster of kFinCtas CTAs per ensemble of up to 512 members; CTA r owns a contiguous
-// block of members from the partials to their ranks. What one member needs from all the
-// others (the mean contour's mass, the calibration scales, the order keys of the depths) is
-// pushed into every CTA's shared memory and separated by cluster barriers, so a finalisation
-// is one launch without tickets or round trips through L2.
+// The members of an ensemble (up to 512) lie in kFinBlocks contiguous blocks. A cluster of C CTAs
+// takes an ensemble, CTA r the blocks r kFinBlocks / C onwards, from the partials to their ranks.
+// What one member needs from all the others (the mean contour's mass, the calibration scales, the
+// order keys of the depths) is pushed into every CTA's shared memory and separated by cluster
+// barriers, so a finalisation is one launch without tickets or round trips through L2.
+//
+// Every sum is ordered by the blocks, never by C: an ensemble's results are the same bits alone
+// and in any batch, whatever C its launch takes.
 //
 // What bounds it is latency: a chain of an L2 read, a few FP64 operations and barriers. GB300
 // issues two FP64 operations per clock and SM, so
@@ -24,12 +27,12 @@ namespace pidk {
 
 namespace {
 
-constexpr int kFinCtas = 8;        // CTAs per ensemble: the portable cluster size
+constexpr int kFinBlocks = 8;      // member blocks, and most CTAs per ensemble: the portable cluster size
 constexpr int kFinThreads = 512;
 constexpr int kFinWarps = kFinThreads / 32;
 constexpr int kFinMaxN = 512;
-constexpr int kFinMaxRows = kFinMaxN / kFinCtas;       // members per CTA
-constexpr int kFinRowsPerWarp = kFinMaxRows / kFinWarps;
+constexpr int kFinMaxRows = kFinMaxN / kFinBlocks;     // members per block
+constexpr int kFinRowsPerWarp = kFinMaxRows / kFinWarps;   // rows that a warp takes at a time
 
 __device__ __forceinline__ const FinDesc& fin_desc(const FinParams& p, int e) {
   return p.descs ? p.descs[e] : p.one;
@@ -42,68 +45,95 @@ __device__ __forceinline__ void fin_sync() {
   else cluster_sync_all();
 }
 
+// Writes v to the shared-memory object at p in each of the ensemble's C CTAs.
+template <int C, typename T>
+__device__ __forceinline__ void fin_push(T* p, T v) {
+  if constexpr (C == 1) {
+    *p = v;
+  } else {
+#pragma unroll
+    for (int r = 0; r < C; ++r) st_cluster(cluster_addr(p, r), v);
+  }
+}
+
 // State shared by the members of one CTA.
+template <int C>
 struct FinShared {
-  float2 acc[kFinThreads];              // partial column sums
-  double tot[2 * kFinMaxRows];          // m of this CTA's members, then N A (or B)
-  double csum[kFinCtas];                // every CTA's share of the mean contour's mass
+  double tot[2][kFinMaxN / C];          // m of this CTA's members; N A (or B)
+  double csum[kFinBlocks];              // every block's share of the mean contour's mass
   unsigned long long key[kFinMaxN];     // order keys of all depths
 };
+// Partial column sums of a CTA's blocks (dynamic shared memory).
+template <int C>
+constexpr size_t fin_acc_bytes() { return sizeof(float2) * kFinThreads * (kFinBlocks / C); }
 
-// Members of one CTA: [m0, m0 + nm), and cp = the power of two that holds ceil(N / CTAs).
+// The power of two that holds n >= 1: its exponent.
+__device__ __forceinline__ int ceil_log2(int n) { return 32 - __clz(n - 1); }
+
+// Members of one CTA: [m0, m0 + nm) in V blocks of `per` members, the first of them block b0; cp =
+// 1 << lg_cp is the power of two that holds a block.
 struct FinSpan {
-  int N, m0, nm, cp;
+  int N, b0, per, m0, nm, lg_cp, cp;
 };
 template <int C>
 __device__ __forceinline__ FinSpan fin_span(int N, int rank) {
+  constexpr int V = kFinBlocks / C;
   FinSpan s;
-  const int per = (N + C - 1) / C;
   s.N = N;
-  s.m0 = min(N, rank * per);
-  s.nm = min(N, s.m0 + per) - s.m0;
-  s.cp = 1;
-  while (s.cp < per) s.cp *= 2;
+  s.b0 = rank * V;
+  s.per = (N + kFinBlocks - 1) / kFinBlocks;
+  s.m0 = min(N, s.b0 * s.per);
+  s.nm = min(N, s.m0 + V * s.per) - s.m0;
+  s.lg_cp = ceil_log2(s.per);
+  s.cp = 1 << s.lg_cp;
   return s;
 }
 
 // Columns of the [rows][2N] partials that belong to this CTA's members into sh.tot: m and
-// N A, or (second) the second half alone. Thread t takes the rows t / columns, + T / columns,
-// ... of one column; the order depends on N and rows alone.
-__device__ void fin_reduce(FinShared& sh, const float* part, int rows, const FinSpan& sp, bool second) {
-  const int ncol = second ? sp.cp : 2 * sp.cp;
-  const int RG = kFinThreads / ncol;
+// N A, or (second) the second half alone. RG row groups take the rows g, g + RG, ... of a column,
+// then the groups of a column are summed. RG, and so the order, depends on N and rows alone: as
+// many groups as give a thread the 8 loads that it keeps in flight, up to one CTA's threads per
+// block.
+template <int C>
+__device__ void fin_reduce(FinShared<C>& sh, float2* acc, const float* part, int rows, const FinSpan& sp,
+                           bool second) {
+  constexpr int V = kFinBlocks / C;
+  const int lg_ncol = sp.lg_cp + (second ? 0 : 1);      // columns of a block, of the CTA
+  const int ncol = 1 << lg_ncol, columns = V * ncol;
+  const int lg_RG = min(ceil_log2((rows + 7) / 8), ceil_log2(kFinThreads) - lg_ncol);
+  const int RG = 1 << lg_RG;
   const int t = threadIdx.x;
   const int64_t stride = 2 * static_cast<int64_t>(sp.N);
-  {
-    const int col = t & (ncol - 1), rg = t / ncol;
-    const int lm = col & (sp.cp - 1);
-    const int half = (second || col >= sp.cp) ? 1 : 0;
+  // the partials of column c, or nullptr for a slot past the CTA's members
+  auto column = [&](int c, int* lm, int* half) -> const float* {
+    const int col = c & (ncol - 1), slot = col & (sp.cp - 1), v = c >> lg_ncol;
+    *half = (second || col >= sp.cp) ? 1 : 0;
+    *lm = v * sp.per + slot;
+    return slot < sp.per && *lm < sp.nm ? part + *half * sp.N + sp.m0 + *lm : nullptr;
+  };
+  for (int e = t; e < columns * RG; e += kFinThreads) {
+    int lm, half;
+    const float* src = column(e & (columns - 1), &lm, &half);
     float2 s = make_float2(0.f, 0.f);
-    if (lm < sp.nm) {
-      const float* src = part + half * sp.N + sp.m0 + lm;
-      int r = rg;
-      for (; r + 7 * RG < rows; r += 8 * RG) {   // 8 loads in flight
+    if (src != nullptr) {
+      for (int r = (e >> lg_ncol) / V; r < rows; r += 8 * RG) {
         float v[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) v[k] = __ldcg(src + (r + k * RG) * stride);
+        for (int k = 0; k < 8; ++k) v[k] = r + k * RG < rows ? __ldcg(src + (r + k * RG) * stride) : 0.f;
 #pragma unroll
         for (int k = 0; k < 8; ++k) pair_add(s, v[k]);
       }
-      float v[7];
-#pragma unroll
-      for (int k = 0; k < 7; ++k) v[k] = r + k * RG < rows ? __ldcg(src + (r + k * RG) * stride) : 0.f;
-#pragma unroll
-      for (int k = 0; k < 7; ++k) pair_add(s, v[k]);
     }
-    sh.acc[t] = s;
+    acc[e] = s;
   }
   __syncthreads();
-  {
-    const int L = min(32, RG);           // lanes that share one column
-    const int c = t / L, l = t & (L - 1);
+  const int lg_L = min(5, lg_RG), L = 1 << lg_L;        // lanes that share one column
+  const int l = t & (L - 1);
+  for (int c0 = 0; c0 < columns; c0 += kFinThreads >> lg_L) {
+    const int c = c0 + (t >> lg_L);
     float2 s = make_float2(0.f, 0.f);
-    if (c < ncol)
-      for (int k = l; k < RG; k += L) pair_add(s, sh.acc[k * ncol + c]);
+    if (c < columns)
+      for (int k = l; k < RG; k += L) pair_add(s, acc[k * columns + c]);
     for (int o = L / 2; o > 0; o >>= 1) {
       const float hi = __shfl_xor_sync(0xffffffffu, s.x, o), lo = __shfl_xor_sync(0xffffffffu, s.y, o);
       // the larger lane index adds the smaller one's value to its own or the other way round:
@@ -113,48 +143,57 @@ __device__ void fin_reduce(FinShared& sh, const float* part, int rows, const Fin
       pair_add(a, (l & o) ? s : other);
       s = a;
     }
-    if (c < ncol && l == 0) {
-      double v = static_cast<double>(s.x) + static_cast<double>(s.y);
-      if (!(fabsf(s.x) <= kMaxFloat)) {       // infinities, NaN, or beyond the FP32 range: in FP64
-        const int lm = c & (sp.cp - 1), half = (second || c >= sp.cp) ? 1 : 0;
-        v = 0.0;
-        if (lm < sp.nm)
-          for (int r = 0; r < rows; ++r)
-            v += static_cast<double>(__ldcg(part + half * sp.N + sp.m0 + lm + r * stride));
+    if (c < columns && l == 0) {
+      int lm, half;
+      const float* src = column(c, &lm, &half);
+      if (src != nullptr) {
+        double v = static_cast<double>(s.x) + static_cast<double>(s.y);
+        if (!(fabsf(s.x) <= kMaxFloat)) {       // infinities, NaN, or beyond the FP32 range: in FP64
+          v = 0.0;
+          for (int r = 0; r < rows; ++r) v += static_cast<double>(__ldcg(src + r * stride));
+        }
+        sh.tot[half][lm] = v;
       }
-      sh.tot[second ? kFinMaxRows + c : (c >= sp.cp ? kFinMaxRows + c - sp.cp : c)] = v;
     }
   }
   __syncthreads();
 }
 
-// The sum of x over all members: every CTA sums its own (xor tree over 64 slots), pushes the
-// result to all CTAs; the cluster barrier that must follow makes csum readable.
+// The blocks' sums of the masses (times the coefficients c, if any), an xor tree over the power of
+// two that holds a block, pushed to all CTAs; the barrier that must follow makes csum readable.
 template <int C>
-__device__ __forceinline__ void fin_push_sum(FinShared& sh, double x_lo, double x_hi, int rank) {
-  if (threadIdx.x < 32) {
-    const double s = warp_sum(x_lo + x_hi);
-    if (threadIdx.x < C) st_cluster(cluster_addr(&sh.csum[rank], threadIdx.x), s);
+__device__ __forceinline__ void fin_push_mass(FinShared<C>& sh, const FinSpan& sp, const float* coef) {
+  constexpr int V = kFinBlocks / C;
+  const int lg = min(sp.lg_cp, 5);                       // 1 << lg lanes of a block, 32 >> lg blocks of a warp
+  const int lane = threadIdx.x & 31, slot = lane & ((1 << lg) - 1);
+  const int v = static_cast<int>(threadIdx.x) >> lg;
+  if ((v & ~((32 >> lg) - 1)) >= V) return;              // the warp's first block
+  auto mass = [&](int x) {
+    const int lm = v * sp.per + x;
+    if (v >= V || x >= sp.per || lm >= sp.nm) return 0.0;
+    return coef ? sh.tot[0][lm] * static_cast<double>(__ldcg(coef + sp.m0 + lm)) : sh.tot[0][lm];
+  };
+  double s = mass(slot);
+  if (sp.lg_cp > 5) s += mass(slot + 32);
+  for (int o = (1 << lg) >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if constexpr (V == 1) {                                // one block: a lane per CTA
+    s = __shfl_sync(0xffffffffu, s, 0);
+    if (lane < C) st_cluster(cluster_addr(&sh.csum[sp.b0], lane), s);
+  } else {
+    if (slot == 0 && v < V) fin_push<C>(&sh.csum[sp.b0 + v], s);
   }
 }
 template <int C>
-__device__ __forceinline__ double fin_total(const FinShared& sh) {
-  if constexpr (C == 1) return sh.csum[0];
-  static_assert(C == 1 || C == 8, "pairwise sum of eight");
+__device__ __forceinline__ double fin_total(const FinShared<C>& sh) {
+  static_assert(kFinBlocks == 8, "pairwise sum of eight");
   return ((sh.csum[0] + sh.csum[1]) + (sh.csum[2] + sh.csum[3])) +
          ((sh.csum[4] + sh.csum[5]) + (sh.csum[6] + sh.csum[7]));
 }
 
-template <int C>
-__device__ __forceinline__ void fin_push_key(FinShared& sh, int i, double depth) {
-  const unsigned long long k = order_key(depth);
-#pragma unroll
-  for (int r = 0; r < C; ++r) st_cluster(cluster_addr(&sh.key[i], r), k);
-}
-
 // Ranks of this CTA's members: one warp per member counts the members that are deeper, or as
 // deep with a lower index.
-__device__ __forceinline__ void fin_ranks(const FinShared& sh, const FinSpan& sp, int32_t* rank) {
+template <int C>
+__device__ __forceinline__ void fin_ranks(const FinShared<C>& sh, const FinSpan& sp, int32_t* rank) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int r = warp; r < sp.nm; r += kFinWarps) {
     const int i = sp.m0 + r;
@@ -174,39 +213,35 @@ __device__ __forceinline__ void fin_ranks(const FinShared& sh, const FinSpan& sp
 // PID-mean, exact full PID and the weighted mean contour. Whole calls against a last CTA that
 // formed the outputs in FP64: 64 x 512^2 fields PID-mean 45.5 -> 33.0 us, 128 x 2^20 exact full
 // PID 215 -> 188 us, of which the finalisation was 15 to 18 us each time.
-__global__ void __cluster_dims__(kFinCtas, 1, 1) __launch_bounds__(kFinThreads, 1)
+template <int C>
+__global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(kFinThreads, 1)
 finalize_kernel(const __grid_constant__ FinParams p) {
-  __shared__ FinShared sh;
-  cluster_arrive();                      // every CTA has started before its memory is written
+  extern __shared__ float2 fin_acc[];
+  __shared__ FinShared<C> sh;
+  if constexpr (C > 1) cluster_arrive(); // every CTA has started before its memory is written
   grid_dependency_wait();
   grid_launch_dependents();              // a second pass may start loading (it waits for this grid's end)
   const FinDesc& d = fin_desc(p, blockIdx.y);
   const int rank = static_cast<int>(blockIdx.x);
-  const FinSpan sp = fin_span<kFinCtas>(d.N, rank);
+  const FinSpan sp = fin_span<C>(d.N, rank);
   const int N = sp.N, t = threadIdx.x;
   const int kind = d.kind;
   const bool wm = kind == FIN_WMEAN, second = kind == FIN_LIN2;
-  fin_reduce(sh, d.part, d.n_chunks, sp, second);
+  fin_reduce<C>(sh, fin_acc, d.part, d.n_chunks, sp, second);
   const int i = sp.m0 + t;
   const bool mine = t < sp.nm;
   double m = 0.0, A = 0.0;               // m_i, N A_i (against a weighted mean contour: A_i)
   if (mine) {
-    m = second ? __ldcg(d.sums + i) : sh.tot[t];
-    A = second ? __ldcg(d.sums + N + i) : sh.tot[kFinMaxRows + t];
+    m = second ? __ldcg(d.sums + i) : sh.tot[0][t];
+    A = second ? __ldcg(d.sums + N + i) : sh.tot[1][t];
   }
-  cluster_wait();
+  if constexpr (C > 1) cluster_wait();
   const bool need_mean = !second && (kind != FIN_LIN1 || d.mean_depth != nullptr);
   double msum = 0.0;
   if (need_mean) {
-    double lo = 0.0, hi = 0.0;
-    if (t < 32) {
-      if (t < sp.nm) lo = wm ? sh.tot[t] * static_cast<double>(__ldcg(d.coef + sp.m0 + t)) : sh.tot[t];
-      if (t + 32 < sp.nm)
-        hi = wm ? sh.tot[t + 32] * static_cast<double>(__ldcg(d.coef + sp.m0 + t + 32)) : sh.tot[t + 32];
-    }
-    fin_push_sum<kFinCtas>(sh, lo, hi, rank);
-    cluster_sync_all();
-    if (mine) msum = fin_total<kFinCtas>(sh);
+    fin_push_mass<C>(sh, sp, wm ? d.coef : nullptr);
+    fin_sync<C>();
+    if (mine) msum = fin_total<C>(sh);
   }
   double depth = 0.0;
   if (mine) {
@@ -224,7 +259,7 @@ finalize_kernel(const __grid_constant__ FinParams p) {
       d.sums[N + i] = A;
       d.coef[i] = m > 0.0 ? static_cast<float>(1.0 / (static_cast<double>(N) * m)) : 0.0f;
     } else {
-      const double in_out = second ? sh.tot[kFinMaxRows + t] : mean_out;
+      const double in_out = second ? sh.tot[1][t] : mean_out;
       depth = fmin(in_in, in_out);
       if (d.depth) d.depth[i] = depth;
       if (d.in_in) d.in_in[i] = in_in;
@@ -232,9 +267,9 @@ finalize_kernel(const __grid_constant__ FinParams p) {
     }
   }
   if (kind != FIN_LIN1 && d.rank != nullptr) {
-    if (mine) fin_push_key<kFinCtas>(sh, i, depth);
-    cluster_sync_all();
-    fin_ranks(sh, sp, d.rank);
+    if (mine) fin_push<C>(&sh.key[i], order_key(depth));
+    fin_sync<C>();
+    fin_ranks<C>(sh, sp, d.rank);
   }
 }
 
@@ -279,12 +314,12 @@ constexpr int kGramSumThreads = 256;
 
 __device__ __forceinline__ float* fin_gram(const FinDesc& d) { return reinterpret_cast<float*>(d.sums + 4 * d.N); }
 
-// Dot products of this warp's rows (warp, warp + 16, ...) of the CTA's [nm][stride] block
-// with the shared vector v: lane l takes the columns l, l + 32, ... in order, then a fixed
-// xor tree.
-__device__ __forceinline__ void rows_dot(const float* C, int stride, int nm, const float* v, int N,
+// Dot products of this warp's rows r0, r0 + 16, ... (kFinRowsPerWarp of them) of the CTA's
+// [nm][stride] block with the shared vector v: lane l takes the columns l, l + 32, ... in order,
+// then a fixed xor tree.
+__device__ __forceinline__ void rows_dot(const float* C, int stride, int r0, int nm, const float* v, int N,
                                          float (&acc)[kFinRowsPerWarp]) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31;
 #pragma unroll
   for (int k = 0; k < kFinRowsPerWarp; ++k) acc[k] = 0.f;
 #pragma unroll 4
@@ -292,7 +327,7 @@ __device__ __forceinline__ void rows_dot(const float* C, int stride, int nm, con
     const float vj = v[j];
 #pragma unroll
     for (int k = 0; k < kFinRowsPerWarp; ++k) {
-      const int r = warp + k * kFinWarps;
+      const int r = r0 + k * kFinWarps;
       if (r < nm) acc[k] = fmaf(C[r * stride + j], vj, acc[k]);
     }
   }
@@ -332,21 +367,22 @@ __global__ void __launch_bounds__(kGramSumThreads) gram_sum_kernel(const __grid_
 // instead of a cluster's (20 x 128^2 BF16 with P: 35.0 -> 30.8 us a call).
 // 512 x 2^20 split BF16 with P: the whole call 2806 -> 2411 us against one CTA that did all of
 // this (437 us); the plume step's three items 1076 -> 996 us (131 us).
-template <int CTAS>
-__global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(kFinThreads, 1)
+template <int C>
+__global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(kFinThreads, 1)
 finalize_gram_kernel(const __grid_constant__ FinParams p) {
-  extern __shared__ float fin_c0[];                     // [nm][N | 1]
-  __shared__ FinShared sh;
+  extern __shared__ float2 fin_acc[];                   // the column sums, then the Gram's rows in their place
+  float* const fin_c0 = reinterpret_cast<float*>(fin_acc);   // [nm][N | 1]
+  __shared__ FinShared<C> sh;
   __shared__ float sd[2][kFinMaxN], sdm[kFinMaxN];      // calibration scales; d_j / m_j
-  __shared__ float starget[kFinMaxRows], sraw[kFinMaxRows];
-  __shared__ int smoved[2][kFinCtas];
-  __shared__ double serr[kFinCtas];
-  if constexpr (CTAS > 1) cluster_arrive();
+  __shared__ float starget[kFinMaxN / C], sraw[kFinMaxN / C];
+  __shared__ int smoved[2][C];
+  __shared__ double serr[C], swarp[kFinWarps];
+  if constexpr (C > 1) cluster_arrive();
   grid_dependency_wait();
   grid_launch_dependents();
   const FinDesc& d = fin_desc(p, blockIdx.y);
   const int rank = static_cast<int>(blockIdx.x);
-  const FinSpan sp = fin_span<CTAS>(d.N, rank);
+  const FinSpan sp = fin_span<C>(d.N, rank);
   const int N = sp.N, t = threadIdx.x, warp = t >> 5, lane = t & 31;
   const int stride = N | 1;
   float* const G = fin_gram(d);
@@ -357,20 +393,13 @@ finalize_gram_kernel(const __grid_constant__ FinParams p) {
       G[col] = gram_chunk_sum(d.gpart + col, d.n_gchunks, NN);
     }
   }
-  fin_reduce(sh, d.part, d.n_chunks, sp, false);
+  fin_reduce<C>(sh, fin_acc, d.part, d.n_chunks, sp, false);
   const int i = sp.m0 + t;
   const bool mine = t < sp.nm;
-  const double m = mine ? sh.tot[t] : 0.0, A = mine ? sh.tot[kFinMaxRows + t] : 0.0;   // m_i, N A_i
-  if constexpr (CTAS > 1) cluster_wait();
-  {
-    double lo = 0.0, hi = 0.0;
-    if (t < 32) {
-      if (t < sp.nm) lo = sh.tot[t];
-      if (t + 32 < sp.nm) hi = sh.tot[t + 32];
-    }
-    fin_push_sum<CTAS>(sh, lo, hi, rank);
-  }
-  fin_sync<CTAS>();    // the other CTAs' shares of the mass; their rows of G (inline sums)
+  const double m = mine ? sh.tot[0][t] : 0.0, A = mine ? sh.tot[1][t] : 0.0;   // m_i, N A_i
+  if constexpr (C > 1) cluster_wait();
+  fin_push_mass<C>(sh, sp, nullptr);
+  fin_sync<C>();       // the other CTAs' shares of the mass; their rows of G (inline sums)
 
   // Row r of the stored array is G'_{., r}, which equals row r of G' up to the rounding of the
   // tensor-core sums: its raw sum, and one half of C0.
@@ -398,7 +427,8 @@ finalize_gram_kernel(const __grid_constant__ FinParams p) {
   }
   __syncthreads();
   {   // ... plus the other half, read across the rows of the other members
-    const int rr = t & (sp.cp - 1), c0 = t / sp.cp, step = kFinThreads / sp.cp;
+    const int lg = sp.nm > 0 ? ceil_log2(sp.nm) : 0;   // threads across this CTA's members
+    const int rr = t & ((1 << lg) - 1), c0 = t >> lg, step = kFinThreads >> lg;
     if (rr < sp.nm) {
       const float* src = G + sp.m0 + rr;
       for (int c = c0; c < N; c += 8 * step) {
@@ -418,7 +448,7 @@ finalize_gram_kernel(const __grid_constant__ FinParams p) {
   }
   double in_in = 0.0, err = 0.0;
   if (mine) {
-    const double msum = fin_total<CTAS>(sh);
+    const double msum = fin_total<C>(sh);
     const double nm_i = m * N;
     in_in = m > 0.0 ? A / nm_i : 0.0;
     if (d.mean_depth) d.mean_depth[i] = fmin(in_in, msum > 0.0 ? A / msum : 0.0);
@@ -427,33 +457,41 @@ finalize_gram_kernel(const __grid_constant__ FinParams p) {
     if (d.err_est) err = m > 0.0 ? fabs(raw / nm_i - in_in) : 0.0;
     starget[t] = static_cast<float>(A);                 // row-sum target N A_i
     const float s0 = (A > 0.0 && raw > 0.0) ? 1.0f : 0.0f;
-#pragma unroll
-    for (int r = 0; r < CTAS; ++r) st_cluster(cluster_addr(&sd[0][i], r), s0);
+    fin_push<C>(&sd[0][i], s0);
   }
-  fin_sync<CTAS>();
+  fin_sync<C>();
+  const int groups = C == kFinBlocks ? 1 : (sp.nm + kFinMaxRows - 1) / kFinMaxRows;   // of rows_dot
   // Symmetric Sinkhorn: d_r <- sqrt(d_r N A_r / sum_j C0_rj d_j), until no scale moves by more
   // than 2^-22 relative (at most 24 sweeps).
   int cur = 0;
   for (int it = 0; it < 24; ++it) {
-    float acc[kFinRowsPerWarp];
-    rows_dot(fin_c0, stride, sp.nm, sd[cur], N, acc);
     bool moved = false;
+    for (int g = 0, r0 = warp; g < groups; ++g, r0 += kFinMaxRows) {
+      float acc[kFinRowsPerWarp];
+      rows_dot(fin_c0, stride, r0, sp.nm, sd[cur], N, acc);
 #pragma unroll
-    for (int k = 0; k < kFinRowsPerWarp; ++k) {
-      const int r = warp + k * kFinWarps;
-      if (r < sp.nm) {
-        const float so = sd[cur][sp.m0 + r];
-        const float sn = (so > 0.f && acc[k] > 0.f) ? sqrtf(so * starget[r] / acc[k]) : 0.f;
-        moved = moved || fabsf(sn - so) > 2.4e-7f * so;
-        if (lane < CTAS) st_cluster(cluster_addr(&sd[cur ^ 1][sp.m0 + r], lane), sn);
+      for (int k = 0; k < kFinRowsPerWarp; ++k) {
+        const int r = r0 + k * kFinWarps;
+        if (r < sp.nm) {
+          const float so = sd[cur][sp.m0 + r];
+          const float sn = (so > 0.f && acc[k] > 0.f) ? sqrtf(so * starget[r] / acc[k]) : 0.f;
+          moved = moved || fabsf(sn - so) > 2.4e-7f * so;
+          if constexpr (C == 1) {
+            if (lane == 0) sd[cur ^ 1][sp.m0 + r] = sn;
+          } else {
+            if (lane < C) st_cluster(cluster_addr(&sd[cur ^ 1][sp.m0 + r], lane), sn);
+          }
+        }
       }
     }
-    const int any = __syncthreads_or(moved);
-    if (t < CTAS) st_cluster(cluster_addr(&smoved[cur][rank], t), any);
-    fin_sync<CTAS>();
-    int more = 0;
+    int more = __syncthreads_or(moved);
+    if constexpr (C > 1) {
+      if (t < C) st_cluster(cluster_addr(&smoved[cur][rank], t), more);
+      cluster_sync_all();
+      more = 0;
 #pragma unroll
-    for (int r = 0; r < CTAS; ++r) more |= smoved[cur][r];
+      for (int r = 0; r < C; ++r) more |= smoved[cur][r];
+    }
     cur ^= 1;
     if (!more) break;
   }
@@ -461,17 +499,16 @@ finalize_gram_kernel(const __grid_constant__ FinParams p) {
   double inv_m = 0.0;
   if (mine) {
     const float dm = m > 0.0 ? static_cast<float>(static_cast<double>(sd[cur][i]) / m) : 0.f;
-#pragma unroll
-    for (int r = 0; r < CTAS; ++r) st_cluster(cluster_addr(&sdm[i], r), dm);
+    fin_push<C>(&sdm[i], dm);
     if (d.P) inv_m = m > 0.0 ? 1.0 / m : 0.0;
   }
-  fin_sync<CTAS>();
-  {
+  fin_sync<C>();
+  for (int g = 0, r0 = warp; g < groups; ++g, r0 += kFinMaxRows) {
     float acc[kFinRowsPerWarp];
-    rows_dot(fin_c0, stride, sp.nm, sdm, N, acc);
+    rows_dot(fin_c0, stride, r0, sp.nm, sdm, N, acc);
 #pragma unroll
     for (int k = 0; k < kFinRowsPerWarp; ++k) {
-      const int r = warp + k * kFinWarps;
+      const int r = r0 + k * kFinWarps;
       if (r < sp.nm && lane == 0) sraw[r] = sd[cur][sp.m0 + r] * acc[k];
     }
   }
@@ -483,43 +520,50 @@ finalize_gram_kernel(const __grid_constant__ FinParams p) {
     if (d.depth) d.depth[i] = depth;
     if (d.in_in) d.in_in[i] = in_in;
     if (d.in_out) d.in_out[i] = in_out;
-    if (d.rank) fin_push_key<CTAS>(sh, i, depth);
-    if (d.P) sh.tot[t] = inv_m;          // 1 / m_i: m is in the owner's registers by now
+    if (d.rank) fin_push<C>(&sh.key[i], order_key(depth));
+    if (d.P) sh.tot[0][t] = inv_m;       // 1 / m_i: m is in the owner's registers by now
   }
   if (d.err_est) {
-    double e = 0.0;
-    if (t < kFinMaxRows) {               // the members sit in the first two warps
+    constexpr int W = kFinMaxN / C / 32;   // warps that can hold members
+    if (warp < W) {
+      if (warp * 32 < sp.nm) {
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) err = fmax(err, __shfl_xor_sync(0xffffffffu, err, o));
-      if (lane == 0) sh.csum[warp] = err;
+        for (int o = 16; o > 0; o >>= 1) err = fmax(err, __shfl_xor_sync(0xffffffffu, err, o));
+      }
+      if (lane == 0) swarp[warp] = err;
     }
     __syncthreads();
-    if (t == 0) {
-      e = fmax(sh.csum[0], sh.csum[1]);
-      st_cluster(cluster_addr(&serr[rank], 0), e);
+    if (warp == 0) {
+      double e = swarp[lane & (W - 1)];
+#pragma unroll
+      for (int o = W / 2; o > 0; o >>= 1) e = fmax(e, __shfl_xor_sync(0xffffffffu, e, o));
+      if (lane == 0) {
+        if constexpr (C == 1) serr[0] = e;
+        else st_cluster(cluster_addr(&serr[rank], 0), e);
+      }
     }
   }
-  fin_sync<CTAS>();
+  fin_sync<C>();
   if (d.err_est && rank == 0 && t == 0) {
     double e = serr[0];
 #pragma unroll
-    for (int r = 1; r < CTAS; ++r) e = fmax(e, serr[r]);
+    for (int r = 1; r < C; ++r) e = fmax(e, serr[r]);
     d.err_est[0] = e;
   }
-  if (d.rank) fin_ranks(sh, sp, d.rank);
+  if (d.rank) fin_ranks<C>(sh, sp, d.rank);
   if (d.P) {
     // P[r][c] = C_rc / m_r. Small ensembles: written here; else C (FP32) and 1 / m_r are
     // stored for gram_matrix_kernel.
     const bool here = N <= kFinInlineMatrixN;
-    float* const C = G + static_cast<int64_t>(N) * N;
+    float* const C0 = G + static_cast<int64_t>(N) * N;
     for (int r = warp; r < sp.nm; r += kFinWarps) {
       const float sr = sd[cur][sp.m0 + r];
-      const double inv = sh.tot[r];
+      const double inv = sh.tot[0][r];
       const int64_t row = static_cast<int64_t>(sp.m0 + r) * N;
       for (int c = lane; c < N; c += 32) {
         const float v = sr * sd[cur][c] * fin_c0[r * stride + c];
         if (here) d.P[row + c] = static_cast<double>(v) * inv;
-        else C[row + c] = v;
+        else C0[row + c] = v;
       }
     }
     if (!here && mine) d.sums[i] = inv_m;
@@ -539,9 +583,26 @@ __global__ void __launch_bounds__(256) gram_matrix_kernel(const __grid_constant_
     d.P[e] = static_cast<double>(__ldcg(C + e)) * __ldcg(d.sums + e / N);
 }
 
+namespace {
+
+constexpr int kFinMaxDynamic = 200 * 1024;   // besides at most 23 KB of static shared memory
+
+// Dynamic shared memory of the Gram's finalisation: its rows, or the column sums before them.
+template <int C>
+size_t fin_gram_smem(int N) {
+  const size_t rows = static_cast<size_t>((N + kFinBlocks - 1) / kFinBlocks) * (kFinBlocks / C);
+  const size_t bytes = rows * (N | 1) * sizeof(float);
+  return bytes > fin_acc_bytes<C>() ? bytes : fin_acc_bytes<C>();
+}
+
+}  // namespace
+
 cudaError_t finalize_kernels_init() {
-  return cudaFuncSetAttribute(finalize_gram_kernel<kFinCtas>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              kFinMaxRows * (kFinMaxN | 1) * static_cast<int>(sizeof(float)));
+  cudaError_t e = cudaFuncSetAttribute(finalize_gram_kernel<kFinBlocks>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       kFinMaxDynamic);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(finalize_gram_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFinMaxDynamic);
+  return e;
 }
 
 namespace {
@@ -565,27 +626,26 @@ cudaError_t fin_launch(K kernel, dim3 grid, int threads, size_t smem, bool pdl, 
 }  // namespace
 
 cudaError_t launch_finalize(const FinParams& p, const FinLaunch& l, cudaStream_t s) {
-  const dim3 grid(kFinCtas, static_cast<unsigned>(l.count));
-  if (!l.gram) return fin_launch(finalize_kernel, grid, kFinThreads, 0, l.pdl, p, s);
+  const unsigned count = static_cast<unsigned>(l.count);
+  if (!l.gram)
+    return fin_launch(finalize_kernel<kFinBlocks>, dim3(kFinBlocks, count), kFinThreads, fin_acc_bytes<kFinBlocks>(),
+                      l.pdl, p, s);
   cudaError_t e = cudaSuccess;
   bool pdl = l.pdl;
   const unsigned NN = static_cast<unsigned>(l.max_n) * static_cast<unsigned>(l.max_n);
   if (l.sum_gram) {
-    e = fin_launch(gram_sum_kernel, dim3((NN + kGramSumThreads - 1) / kGramSumThreads, grid.y),
+    e = fin_launch(gram_sum_kernel, dim3((NN + kGramSumThreads - 1) / kGramSumThreads, count),
                    kGramSumThreads, 0, pdl, p, s);
     if (e != cudaSuccess) return e;
     pdl = true;
   }
-  if (l.single) {
-    const size_t smem = static_cast<size_t>(l.max_n) * (l.max_n | 1) * sizeof(float);
-    e = fin_launch(finalize_gram_kernel<1>, dim3(1, grid.y), kFinThreads, smem, pdl, p, s);
-    if (e != cudaSuccess || !l.matrix) return e;
-    return fin_launch(gram_matrix_kernel, dim3((NN + 1023) / 1024, grid.y), 256, 0, true, p, s);
-  }
-  const size_t rows = (static_cast<size_t>(l.max_n) + kFinCtas - 1) / kFinCtas;
-  e = fin_launch(finalize_gram_kernel<kFinCtas>, grid, kFinThreads, rows * (l.max_n | 1) * sizeof(float), pdl, p, s);
+  if (l.single)
+    e = fin_launch(finalize_gram_kernel<1>, dim3(1, count), kFinThreads, fin_gram_smem<1>(l.max_n), pdl, p, s);
+  else
+    e = fin_launch(finalize_gram_kernel<kFinBlocks>, dim3(kFinBlocks, count), kFinThreads,
+                   fin_gram_smem<kFinBlocks>(l.max_n), pdl, p, s);
   if (e != cudaSuccess || !l.matrix) return e;
-  return fin_launch(gram_matrix_kernel, dim3((NN + 1023) / 1024, grid.y), 256, 0, true, p, s);
+  return fin_launch(gram_matrix_kernel, dim3((NN + 1023) / 1024, count), 256, 0, true, p, s);
 }
 
 }  // namespace pidk
