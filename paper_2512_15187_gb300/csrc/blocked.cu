@@ -154,28 +154,28 @@ struct LargeFin {
   double *depth, *in_in, *in_out, *mass, *mean_depth;
 };
 
-// Column i of the partials summed over this thread's rows (FP32 pairs, see pair_add).
-__device__ __forceinline__ float2 large_column(const float* src, int64_t stride, int rows, int r0) {
-  float2 s = make_float2(0.f, 0.f);
+// Column i of the partials summed over this thread's rows.
+__device__ __forceinline__ Sum3 large_column(const float* src, int64_t stride, int rows, int r0) {
+  Sum3 s;
   int r = r0;
   for (; r + 3 * kLargeRows < rows; r += 4 * kLargeRows) {
     float v[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) v[k] = __ldcg(src + (r + k * kLargeRows) * stride);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) pair_add(s, v[k]);
+    for (int k = 0; k < 4; ++k) sum3_add(s, v[k]);
   }
-  for (; r < rows; r += kLargeRows) pair_add(s, __ldcg(src + r * stride));
+  for (; r < rows; r += kLargeRows) sum3_add(s, __ldcg(src + r * stride));
   return s;
 }
 
 // The sum of a column's row groups in FP64; sums that leave the finite FP32 range again in FP64.
-__device__ __forceinline__ double large_total(const float2 (*acc)[kLargeMembers], int lane,
+__device__ __forceinline__ double large_total(const Sum3 (*acc)[kLargeMembers], int lane,
                                               const float* src, int64_t stride, int rows) {
-  float2 s = acc[0][lane];
+  Sum3 s = acc[0][lane];
 #pragma unroll
-  for (int g = 1; g < kLargeRows; ++g) pair_add(s, acc[g][lane]);
-  if (fabsf(s.x) <= kMaxFloat) return static_cast<double>(s.x) + static_cast<double>(s.y);
+  for (int g = 1; g < kLargeRows; ++g) sum3_add(s, acc[g][lane]);
+  if (fabsf(s.x) <= kMaxFloat) return sum3_value(s);
   double v = 0.0;
   for (int r = 0; r < rows; ++r) v += static_cast<double>(__ldcg(src + r * stride));
   return v;
@@ -185,14 +185,14 @@ __device__ __forceinline__ double large_total(const float2 (*acc)[kLargeMembers]
 // added by the last CTA in order. (One CTA used to form every member's outputs as well, with
 // FP64 divisions at two operations per clock: 107 us for 10 000 members.)
 __global__ void __launch_bounds__(kLargeThreads) large_sum_kernel(const __grid_constant__ LargeFin p) {
-  __shared__ float2 acc[2][kLargeRows][kLargeMembers];
+  __shared__ Sum3 acc[2][kLargeRows][kLargeMembers];
   __shared__ double red[kLargeThreads];
   __shared__ bool last;
   const int lane = threadIdx.x & 31, rg = threadIdx.x >> 5;
   const int64_t i = static_cast<int64_t>(blockIdx.x) * kLargeMembers + lane;
   const int64_t stride = 2 * p.N;
   const bool second = p.kind == FIN_LIN2, in = i < p.N;
-  const float2 zero = make_float2(0.f, 0.f);
+  const Sum3 zero{};
   acc[0][rg][lane] = in && !second ? large_column(p.part + i, stride, p.n_chunks, rg) : zero;
   acc[1][rg][lane] = in ? large_column(p.part + p.N + i, stride, p.n_chunks, rg) : zero;
   __syncthreads();

@@ -254,16 +254,29 @@ __device__ __forceinline__ double warp_sum(double v) {
 
 constexpr float kMaxFloat = 3.402823466e38f;   // largest finite FP32
 
-// hi + lo += x, with the rounding error of the FP32 addition kept in lo (2Sum, Knuth).
-__device__ __forceinline__ void pair_add(float2& s, float x) {
-  const float t = s.x + x;
-  const float b = t - s.x;
-  s.y += (s.x - (t - b)) + (x - b);
-  s.x = t;
+// A sum of FP32 values as an unevaluated sum of three: x is the running FP32 sum, y that of its
+// rounding errors, z that of the errors of y (2Sum, Knuth, at both levels), so that what is lost
+// lies some 70 bits below the sum (of up to 2^13 values) and its FP64 value is good to the last bit
+// but one. 13 FP32 operations a value: GB300 has 64 times as many FP32 as FP64 lanes.
+struct Sum3 {
+  float x = 0.f, y = 0.f, z = 0.f;
+};
+// a + b -> a; returns the rounding error.
+__device__ __forceinline__ float two_sum(float& a, float b) {
+  const float t = a + b;
+  const float v = t - a;
+  const float e = (a - (t - v)) + (b - v);
+  a = t;
+  return e;
 }
-__device__ __forceinline__ void pair_add(float2& s, float2 v) {
-  pair_add(s, v.x);
-  s.y += v.y;
+__device__ __forceinline__ void sum3_add(Sum3& s, float v) { s.z += two_sum(s.y, two_sum(s.x, v)); }
+__device__ __forceinline__ void sum3_add(Sum3& s, const Sum3& v) {
+  sum3_add(s, v.x);
+  s.z += two_sum(s.y, v.y);
+  s.z += v.z;
+}
+__device__ __forceinline__ double sum3_value(const Sum3& s) {
+  return static_cast<double>(s.x) + (static_cast<double>(s.y) + static_cast<double>(s.z));
 }
 
 // Order-preserving integer key of a double: for non-NaN a, b, a < b <=> key(a) < key(b) and

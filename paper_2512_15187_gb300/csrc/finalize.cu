@@ -13,9 +13,9 @@
 //
 // What bounds it is latency: a chain of an L2 read, a few FP64 operations and barriers. GB300
 // issues two FP64 operations per clock and SM, so
-//   * the partials, which are FP32 values, are summed as unevaluated FP32 pairs (2Sum: the sum's
-//     rounding errors are carried along, about 48 significant bits) and become FP64 once per
-//     column; a sum that leaves the finite FP32 range is formed again in FP64;
+//   * the partials, which are FP32 values, are summed as unevaluated sums of three FP32 numbers
+//     (Sum3: what is lost lies below FP64's last bit) and become FP64 once per column; a sum that
+//     leaves the finite FP32 range is formed again in FP64;
 //   * the FP64 divisions and the N^2 rank comparisons are spread over the cluster's SMs.
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -65,7 +65,7 @@ struct FinShared {
 };
 // Partial column sums of a CTA's blocks (dynamic shared memory).
 template <int C>
-constexpr size_t fin_acc_bytes() { return sizeof(float2) * kFinThreads * (kFinBlocks / C); }
+constexpr size_t fin_acc_bytes() { return sizeof(Sum3) * kFinThreads * (kFinBlocks / C); }
 
 // The power of two that holds n >= 1: its exponent.
 __device__ __forceinline__ int ceil_log2(int n) { return 32 - __clz(n - 1); }
@@ -95,7 +95,7 @@ __device__ __forceinline__ FinSpan fin_span(int N, int rank) {
 // many groups as give a thread the 8 loads that it keeps in flight, up to one CTA's threads per
 // block.
 template <int C>
-__device__ void fin_reduce(FinShared<C>& sh, float2* acc, const float* part, int rows, const FinSpan& sp,
+__device__ void fin_reduce(FinShared<C>& sh, Sum3* acc, const float* part, int rows, const FinSpan& sp,
                            bool second) {
   constexpr int V = kFinBlocks / C;
   const int lg_ncol = sp.lg_cp + (second ? 0 : 1);      // columns of a block, of the CTA
@@ -114,14 +114,24 @@ __device__ void fin_reduce(FinShared<C>& sh, float2* acc, const float* part, int
   for (int e = t; e < columns * RG; e += kFinThreads) {
     int lm, half;
     const float* src = column(e & (columns - 1), &lm, &half);
-    float2 s = make_float2(0.f, 0.f);
+    Sum3 s;
     if (src != nullptr) {
-      for (int r = (e >> lg_ncol) / V; r < rows; r += 8 * RG) {
-        float v[8];
+      // the next 8 rows are in flight while these are added (an addition costs 13 instructions)
+      float v[8], w[8];
+      auto load = [&](float (&x)[8], int r) {
 #pragma unroll
-        for (int k = 0; k < 8; ++k) v[k] = r + k * RG < rows ? __ldcg(src + (r + k * RG) * stride) : 0.f;
+        for (int k = 0; k < 8; ++k) x[k] = r + k * RG < rows ? __ldcg(src + (r + k * RG) * stride) : 0.f;
+      };
+      int r = (e >> lg_ncol) / V;
+      load(v, r);
+      while (r < rows) {
+        load(w, r + 8 * RG);
 #pragma unroll
-        for (int k = 0; k < 8; ++k) pair_add(s, v[k]);
+        for (int k = 0; k < 8; ++k)
+          sum3_add(s, v[k]);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = w[k];
+        r += 8 * RG;
       }
     }
     acc[e] = s;
@@ -131,30 +141,34 @@ __device__ void fin_reduce(FinShared<C>& sh, float2* acc, const float* part, int
   const int l = t & (L - 1);
   for (int c0 = 0; c0 < columns; c0 += kFinThreads >> lg_L) {
     const int c = c0 + (t >> lg_L);
-    float2 s = make_float2(0.f, 0.f);
+    Sum3 s;
     if (c < columns)
-      for (int k = l; k < RG; k += L) pair_add(s, acc[k * columns + c]);
+      for (int k = l; k < RG; k += L) sum3_add(s, acc[k * columns + c]);
     for (int o = L / 2; o > 0; o >>= 1) {
-      const float hi = __shfl_xor_sync(0xffffffffu, s.x, o), lo = __shfl_xor_sync(0xffffffffu, s.y, o);
+      Sum3 other;
+      other.x = __shfl_xor_sync(0xffffffffu, s.x, o);
+      other.y = __shfl_xor_sync(0xffffffffu, s.y, o);
+      other.z = __shfl_xor_sync(0xffffffffu, s.z, o);
       // the larger lane index adds the smaller one's value to its own or the other way round:
-      // both lanes form the same sum because the lower lane's pair always comes first
-      const float2 other = make_float2(hi, lo);
-      float2 a = (l & o) ? other : s;
-      pair_add(a, (l & o) ? s : other);
+      // both lanes form the same sum because the lower lane's always comes first
+      Sum3 a = (l & o) ? other : s;
+      sum3_add(a, (l & o) ? s : other);
       s = a;
     }
-    if (c < columns && l == 0) {
-      int lm, half;
-      const float* src = column(c, &lm, &half);
-      if (src != nullptr) {
-        double v = static_cast<double>(s.x) + static_cast<double>(s.y);
-        if (!(fabsf(s.x) <= kMaxFloat)) {       // infinities, NaN, or beyond the FP32 range: in FP64
-          v = 0.0;
-          for (int r = 0; r < rows; ++r) v += static_cast<double>(__ldcg(src + r * stride));
-        }
-        sh.tot[half][lm] = v;
-      }
+    if (c < columns && l == 0) acc[c] = s;      // in place of the group 0 that this lane alone read
+  }
+  __syncthreads();
+  // to FP64 with a thread per column (few warps: the FP64 pipe takes 16 clocks an instruction)
+  for (int c = t; c < columns; c += kFinThreads) {
+    int lm, half;
+    const float* src = column(c, &lm, &half);
+    if (src == nullptr) continue;
+    double v = sum3_value(acc[c]);
+    if (!(fabsf(acc[c].x) <= kMaxFloat)) {      // infinities, NaN, or beyond the FP32 range: in FP64
+      v = 0.0;
+      for (int r = 0; r < rows; ++r) v += static_cast<double>(__ldcg(src + r * stride));
     }
+    sh.tot[half][lm] = v;
   }
   __syncthreads();
 }
@@ -216,7 +230,7 @@ __device__ __forceinline__ void fin_ranks(const FinShared<C>& sh, const FinSpan&
 template <int C>
 __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(kFinThreads, 1)
 finalize_kernel(const __grid_constant__ FinParams p) {
-  extern __shared__ float2 fin_acc[];
+  extern __shared__ float fin_dyn[];
   __shared__ FinShared<C> sh;
   if constexpr (C > 1) cluster_arrive(); // every CTA has started before its memory is written
   grid_dependency_wait();
@@ -227,7 +241,7 @@ finalize_kernel(const __grid_constant__ FinParams p) {
   const int N = sp.N, t = threadIdx.x;
   const int kind = d.kind;
   const bool wm = kind == FIN_WMEAN, second = kind == FIN_LIN2;
-  fin_reduce<C>(sh, fin_acc, d.part, d.n_chunks, sp, second);
+  fin_reduce<C>(sh, reinterpret_cast<Sum3*>(fin_dyn), d.part, d.n_chunks, sp, second);
   const int i = sp.m0 + t;
   const bool mine = t < sp.nm;
   double m = 0.0, A = 0.0;               // m_i, N A_i (against a weighted mean contour: A_i)
@@ -370,8 +384,8 @@ __global__ void __launch_bounds__(kGramSumThreads) gram_sum_kernel(const __grid_
 template <int C>
 __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(kFinThreads, 1)
 finalize_gram_kernel(const __grid_constant__ FinParams p) {
-  extern __shared__ float2 fin_acc[];                   // the column sums, then the Gram's rows in their place
-  float* const fin_c0 = reinterpret_cast<float*>(fin_acc);   // [nm][N | 1]
+  extern __shared__ float fin_dyn[];
+  float* const fin_c0 = fin_dyn;                        // [nm][N | 1], where the column sums were before
   __shared__ FinShared<C> sh;
   __shared__ float sd[2][kFinMaxN], sdm[kFinMaxN];      // calibration scales; d_j / m_j
   __shared__ float starget[kFinMaxN / C], sraw[kFinMaxN / C];
@@ -393,7 +407,7 @@ finalize_gram_kernel(const __grid_constant__ FinParams p) {
       G[col] = gram_chunk_sum(d.gpart + col, d.n_gchunks, NN);
     }
   }
-  fin_reduce<C>(sh, fin_acc, d.part, d.n_chunks, sp, false);
+  fin_reduce<C>(sh, reinterpret_cast<Sum3*>(fin_dyn), d.part, d.n_chunks, sp, false);
   const int i = sp.m0 + t;
   const bool mine = t < sp.nm;
   const double m = mine ? sh.tot[0][t] : 0.0, A = mine ? sh.tot[1][t] : 0.0;   // m_i, N A_i
