@@ -640,8 +640,8 @@ static pid_status enqueue(pid_handle h, const BatchPlan& bp, char* base, const v
         e = cudaEventRecord(c->fork_ev, s);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(sg, c->fork_ev, 0);
       }
-      if (e == cudaSuccess && l1.count) e = launch_finalize(fg, l1, sg);
-      if (e == cudaSuccess && l0.count) e = launch_finalize(fp, l0, s);
+      if (e == cudaSuccess && l1.count) e = launch_finalize(fg, l1, h->sms, sg);
+      if (e == cudaSuccess && l0.count) e = launch_finalize(fp, l0, h->sms, s);
       if (e == cudaSuccess && fork) {
         e = cudaEventRecord(c->join_ev[0], sg);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(s, c->join_ev[0], 0);

@@ -606,7 +606,7 @@ pid_status launch_fin_one(pid_handle h, const FinDesc& fd, cudaStream_t s) {
   fp.n_ens = 1;
   fp.err = h->err_word;
   ProfScope ps(h, PID_KERNEL_FINALIZE, 0.0, 0.0, s);
-  cudaError_t e = launch_finalize(fp, l, s);
+  cudaError_t e = launch_finalize(fp, l, h->sms, s);
   if (e != cudaSuccess) return cuda_fail(h, e, "finalize launch");
   return PID_OK;
 }

@@ -271,9 +271,8 @@ __device__ __forceinline__ float two_sum(float& a, float b) {
 }
 __device__ __forceinline__ void sum3_add(Sum3& s, float v) { s.z += two_sum(s.y, two_sum(s.x, v)); }
 __device__ __forceinline__ void sum3_add(Sum3& s, const Sum3& v) {
-  sum3_add(s, v.x);
-  s.z += two_sum(s.y, v.y);
-  s.z += v.z;
+  const float e = two_sum(s.x, v.x), f = two_sum(s.y, v.y);
+  s.z = (s.z + v.z) + (f + two_sum(s.y, e));
 }
 __device__ __forceinline__ double sum3_value(const Sum3& s) {
   return static_cast<double>(s.x) + (static_cast<double>(s.y) + static_cast<double>(s.z));

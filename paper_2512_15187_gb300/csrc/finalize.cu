@@ -127,8 +127,7 @@ __device__ void fin_reduce(FinShared<C>& sh, Sum3* acc, const float* part, int r
       while (r < rows) {
         load(w, r + 8 * RG);
 #pragma unroll
-        for (int k = 0; k < 8; ++k)
-          sum3_add(s, v[k]);
+        for (int k = 0; k < 8; ++k) sum3_add(s, v[k]);
 #pragma unroll
         for (int k = 0; k < 8; ++k) v[k] = w[k];
         r += 8 * RG;
@@ -139,25 +138,21 @@ __device__ void fin_reduce(FinShared<C>& sh, Sum3* acc, const float* part, int r
   __syncthreads();
   const int lg_L = min(5, lg_RG), L = 1 << lg_L;        // lanes that share one column
   const int l = t & (L - 1);
-  for (int c0 = 0; c0 < columns; c0 += kFinThreads >> lg_L) {
+  for (int c0 = 0; L > 1 && c0 < columns; c0 += kFinThreads >> lg_L) {
     const int c = c0 + (t >> lg_L);
     Sum3 s;
     if (c < columns)
       for (int k = l; k < RG; k += L) sum3_add(s, acc[k * columns + c]);
-    for (int o = L / 2; o > 0; o >>= 1) {
+    for (int o = L / 2; o > 0; o >>= 1) {     // tree: lane 0 ends with the column's sum
       Sum3 other;
       other.x = __shfl_xor_sync(0xffffffffu, s.x, o);
       other.y = __shfl_xor_sync(0xffffffffu, s.y, o);
       other.z = __shfl_xor_sync(0xffffffffu, s.z, o);
-      // the larger lane index adds the smaller one's value to its own or the other way round:
-      // both lanes form the same sum because the lower lane's always comes first
-      Sum3 a = (l & o) ? other : s;
-      sum3_add(a, (l & o) ? s : other);
-      s = a;
+      sum3_add(s, other);
     }
-    if (c < columns && l == 0) acc[c] = s;      // in place of the group 0 that this lane alone read
+    if (c < columns && l == 0) acc[c] = s;    // in place of the group 0 that this lane alone read
   }
-  __syncthreads();
+  if (L > 1) __syncthreads();
   // to FP64 with a thread per column (few warps: the FP64 pipe takes 16 clocks an instruction)
   for (int c = t; c < columns; c += kFinThreads) {
     int lm, half;
@@ -228,7 +223,7 @@ __device__ __forceinline__ void fin_ranks(const FinShared<C>& sh, const FinSpan&
 // formed the outputs in FP64: 64 x 512^2 fields PID-mean 45.5 -> 33.0 us, 128 x 2^20 exact full
 // PID 215 -> 188 us, of which the finalisation was 15 to 18 us each time.
 template <int C>
-__global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(kFinThreads, 1)
+__global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(kFinThreads, 2)
 finalize_kernel(const __grid_constant__ FinParams p) {
   extern __shared__ float fin_dyn[];
   __shared__ FinShared<C> sh;
@@ -381,8 +376,8 @@ __global__ void __launch_bounds__(kGramSumThreads) gram_sum_kernel(const __grid_
 // instead of a cluster's (20 x 128^2 BF16 with P: 35.0 -> 30.8 us a call).
 // 512 x 2^20 split BF16 with P: the whole call 2806 -> 2411 us against one CTA that did all of
 // this (437 us); the plume step's three items 1076 -> 996 us (131 us).
-template <int C>
-__global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(kFinThreads, 1)
+template <int C, int PER_SM>
+__global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(kFinThreads, PER_SM)
 finalize_gram_kernel(const __grid_constant__ FinParams p) {
   extern __shared__ float fin_dyn[];
   float* const fin_c0 = fin_dyn;                        // [nm][N | 1], where the column sums were before
@@ -600,22 +595,36 @@ __global__ void __launch_bounds__(256) gram_matrix_kernel(const __grid_constant_
 namespace {
 
 constexpr int kFinMaxDynamic = 200 * 1024;   // besides at most 23 KB of static shared memory
+constexpr int kFinTwoDynamic = 88 * 1024;    // so that two CTAs fit an SM
 
 // Dynamic shared memory of the Gram's finalisation: its rows, or the column sums before them.
 template <int C>
-size_t fin_gram_smem(int N) {
+constexpr size_t fin_gram_smem(int N) {
   const size_t rows = static_cast<size_t>((N + kFinBlocks - 1) / kFinBlocks) * (kFinBlocks / C);
   const size_t bytes = rows * (N | 1) * sizeof(float);
   return bytes > fin_acc_bytes<C>() ? bytes : fin_acc_bytes<C>();
 }
 
+template <int C>
+cudaError_t fin_init() {
+  cudaError_t e = cudaFuncSetAttribute(finalize_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       static_cast<int>(fin_acc_bytes<C>()));
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(finalize_gram_kernel<C, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFinMaxDynamic);
+  if constexpr (C < kFinBlocks) {
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(finalize_gram_kernel<C, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFinTwoDynamic);
+  }
+  return e;
+}
+
 }  // namespace
 
 cudaError_t finalize_kernels_init() {
-  cudaError_t e = cudaFuncSetAttribute(finalize_gram_kernel<kFinBlocks>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       kFinMaxDynamic);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(finalize_gram_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFinMaxDynamic);
+  cudaError_t e = fin_init<1>();
+  if (e == cudaSuccess) e = fin_init<2>();
+  if (e == cudaSuccess) e = fin_init<4>();
+  if (e == cudaSuccess) e = fin_init<8>();
   return e;
 }
 
@@ -637,15 +646,59 @@ cudaError_t fin_launch(K kernel, dim3 grid, int threads, size_t smem, bool pdl, 
   return cudaLaunchKernelEx(&cfg, kernel, p);
 }
 
+// The launch with C CTAs per ensemble if `force`, or if all of them are on the GPU at once; sets `done`
+// if it was made. Ensembles that fill less than the SMs get one each: two on an SM are slower than
+// one (the Gram is compiled for either, with 80 and 64 registers: 50 x (32 x 4096) 53.6 and 49.5 us).
+template <int C>
+cudaError_t fin_try(const FinParams& p, const FinLaunch& l, int sms, bool pdl, bool force, bool* done, cudaStream_t s) {
+  if (*done) return cudaSuccess;
+  const int64_t ctas = static_cast<int64_t>(l.count) * C;
+  const dim3 grid(C, static_cast<unsigned>(l.count));
+  if (!l.gram) {
+    if (!force && ctas > 2 * sms) return cudaSuccess;
+    *done = true;
+    return fin_launch(finalize_kernel<C>, grid, kFinThreads, fin_acc_bytes<C>(), pdl, p, s);
+  }
+  const size_t smem = fin_gram_smem<C>(l.max_n);
+  if (smem > kFinMaxDynamic) return cudaSuccess;
+  if constexpr (C < kFinBlocks) {
+    const bool two = smem <= kFinTwoDynamic;
+    if (ctas > sms && two && (force || ctas <= 2 * sms)) {
+      *done = true;
+      return fin_launch(finalize_gram_kernel<C, 2>, grid, kFinThreads, smem, pdl, p, s);
+    }
+  }
+  if (!force && ctas > sms) return cudaSuccess;
+  *done = true;
+  return fin_launch(finalize_gram_kernel<C, 1>, grid, kFinThreads, smem, pdl, p, s);
+}
+
+// CTAs per ensemble: the most that let every ensemble start at once. An ensemble's chain of barriers
+// and round trips gets shorter with more CTAs, but a second wave of ensembles waits for all of the
+// first one's. More ensembles than that take one CTA each (Gram: the fewest that hold its rows).
+// Batches, eight CTAs each -> this rule: PID-mean of 1000 x (8 x 1024) 198 -> 51 us, of 200 x
+// (20 x 16 384) 149 -> 123; BF16 Gram of 200 x (64 x 4096) 369 -> 123, of 50 x (200 x 8192) 321 -> 264.
+cudaError_t fin_launch_ctas(const FinParams& p, const FinLaunch& l, int sms, bool pdl, cudaStream_t s) {
+  bool done = false;
+  cudaError_t e = cudaSuccess;
+  if (!(l.gram && l.single)) {
+    e = fin_try<8>(p, l, sms, pdl, false, &done, s);
+    if (e == cudaSuccess) e = fin_try<4>(p, l, sms, pdl, false, &done, s);
+    if (e == cudaSuccess) e = fin_try<2>(p, l, sms, pdl, false, &done, s);
+  }
+  if (e == cudaSuccess) e = fin_try<1>(p, l, sms, pdl, true, &done, s);
+  if (e == cudaSuccess) e = fin_try<2>(p, l, sms, pdl, true, &done, s);
+  if (e == cudaSuccess) e = fin_try<4>(p, l, sms, pdl, true, &done, s);
+  if (e == cudaSuccess) e = fin_try<8>(p, l, sms, pdl, true, &done, s);
+  return e;
+}
+
 }  // namespace
 
-cudaError_t launch_finalize(const FinParams& p, const FinLaunch& l, cudaStream_t s) {
-  const unsigned count = static_cast<unsigned>(l.count);
-  if (!l.gram)
-    return fin_launch(finalize_kernel<kFinBlocks>, dim3(kFinBlocks, count), kFinThreads, fin_acc_bytes<kFinBlocks>(),
-                      l.pdl, p, s);
+cudaError_t launch_finalize(const FinParams& p, const FinLaunch& l, int sms, cudaStream_t s) {
   cudaError_t e = cudaSuccess;
   bool pdl = l.pdl;
+  const unsigned count = static_cast<unsigned>(l.count);
   const unsigned NN = static_cast<unsigned>(l.max_n) * static_cast<unsigned>(l.max_n);
   if (l.sum_gram) {
     e = fin_launch(gram_sum_kernel, dim3((NN + kGramSumThreads - 1) / kGramSumThreads, count),
@@ -653,11 +706,7 @@ cudaError_t launch_finalize(const FinParams& p, const FinLaunch& l, cudaStream_t
     if (e != cudaSuccess) return e;
     pdl = true;
   }
-  if (l.single)
-    e = fin_launch(finalize_gram_kernel<1>, dim3(1, count), kFinThreads, fin_gram_smem<1>(l.max_n), pdl, p, s);
-  else
-    e = fin_launch(finalize_gram_kernel<kFinBlocks>, dim3(kFinBlocks, count), kFinThreads,
-                   fin_gram_smem<kFinBlocks>(l.max_n), pdl, p, s);
+  e = fin_launch_ctas(p, l, sms, pdl, s);
   if (e != cudaSuccess || !l.matrix) return e;
   return fin_launch(gram_matrix_kernel, dim3((NN + 1023) / 1024, count), 256, 0, true, p, s);
 }

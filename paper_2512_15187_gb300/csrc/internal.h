@@ -265,7 +265,7 @@ inline int iso_kind(int32_t iso_mode) { return iso_mode == ISO_NONE ? 0 : (iso_m
 
 cudaError_t launch_stream(const StreamParams& p, int vec, int mpw, int G, int iso_kind, bool coef,
                           int grid, size_t smem, cudaStream_t s);
-cudaError_t launch_finalize(const FinParams& p, const FinLaunch& l, cudaStream_t s);   // finalize.cu
+cudaError_t launch_finalize(const FinParams& p, const FinLaunch& l, int sms, cudaStream_t s);   // finalize.cu
 cudaError_t finalize_kernels_init();
 cudaError_t launch_iso(const IsoParams& p, cudaStream_t s);
 cudaError_t launch_member_coef(const double* r, int64_t N, float* coef, uint32_t* err,

@@ -140,7 +140,7 @@ extern "C" pid_status pid_mean_noalloc(const float* U, int64_t N, int64_t M, int
   FinLaunch fl;
   pidh::fin_launch_add(&fl, fd);
   fl.pdl = true;
-  if (launch_finalize(fp, fl, s) != cudaSuccess) return PID_ERR_CUDA;
+  if (launch_finalize(fp, fl, ds->sms, s) != cudaSuccess) return PID_ERR_CUDA;
   if (device_status &&
       cudaMemcpyAsync(device_status, err_word, sizeof(uint32_t), cudaMemcpyDeviceToDevice, s) !=
           cudaSuccess)

@@ -85,3 +85,15 @@ def test_served_mix(H):
                     np.testing.assert_array_equal(o[f], to_np(alone[k][f]), err_msg=f"{SHAPES[k]} {f}")
     finally:
         srv.stop()
+
+
+# eight, four, two and one CTA per ensemble (152 SMs); 256 members' rows need two
+@pytest.mark.parametrize("count", [10, 30, 60, 120, 320])
+@pytest.mark.parametrize("N,M", [(33, 6000), (100, 4096), (225, 2048), (256, 2048)])
+def test_many_gram_items(H, count, N, M):
+    U = _dev(_masks(N, M))
+    alone = H.full(U, mode="full", precision="split_bf16", want_P=True)
+    outs = H.batch([dict(data=U, mode="full", precision="split_bf16", want_P=True)] * count)
+    H.sync()
+    for o in outs:
+        _same(o, alone, f"{N} x {M}, {count} items")
