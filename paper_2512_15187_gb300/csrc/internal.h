@@ -241,6 +241,7 @@ struct IsoParams {
   int32_t iso_mode;
   float iso_mu, iso_inv, iso_t;
   int32_t out_bf16;
+  int32_t lg_row;          // set by launch_iso: 1 << lg_row threads per row
 };
 
 // The Gram partials of small ensembles are summed by the finalisation's own CTAs (a launch

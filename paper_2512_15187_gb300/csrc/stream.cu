@@ -167,49 +167,62 @@ __device__ __forceinline__ float4 iso_map4(const float4& f, const IsoParams& p) 
 
 // HBM-bound: 4 B read and 4 (2) B written per element. Rows lie along the grid's y axis, so no
 // element divides its index; contiguous ensembles come as one row, whatever M is. VEC: rows
-// aligned for 4-element accesses, four of them in flight per thread; else element by element.
+// aligned for 4-element accesses; else element by element. A thread has four accesses in flight:
+// along its row, a CTA per row, or (SHORT) one each in four rows, 1 << lg_row threads to a row.
 // 64 fields of 2048^2 cells to FP32: 0.453 -> 0.304 ms (7.1 TB/s) against one element group per
-// grid-stride step with a 64-bit division.
-template <bool BF16, int KIND, bool VEC>
+// grid-stride step with a 64-bit division; 100 000 rows of 16 cells, 32 apart: 114 -> 16 us against
+// a CTA per row.
+template <bool BF16, int KIND, bool VEC, bool SHORT>
 __global__ void __launch_bounds__(kIsoThreads) iso_kernel(const __grid_constant__ IsoParams p) {
-  constexpr int64_t kTile = static_cast<int64_t>(kIsoThreads) * kIsoUnroll * (VEC ? 4 : 1);
-  const int64_t x0 = blockIdx.x * kTile;
-  for (int64_t i = blockIdx.y; i < p.N; i += gridDim.y) {
-    const float* src = p.F + i * p.ld;
-    const int64_t row = i * p.ld_out;
+  constexpr int W = VEC ? 4 : 1;
+  const int rows = SHORT ? kIsoThreads >> p.lg_row : 1;              // side by side in the CTA
+  const int t = SHORT ? static_cast<int>(threadIdx.x) & ((1 << p.lg_row) - 1) : static_cast<int>(threadIdx.x);
+  const int64_t x0 = SHORT ? t * W : static_cast<int64_t>(blockIdx.x) * kIsoThreads * kIsoUnroll * W + t * W;
+  const int64_t step = SHORT ? int64_t(rows) * kIsoUnroll : 1;       // rows of the CTA at a time
+  auto cell = [&](int u) { return SHORT ? x0 : x0 + static_cast<int64_t>(u) * kIsoThreads * W; };
+  for (int64_t i0 = blockIdx.y * step + (SHORT ? threadIdx.x >> p.lg_row : 0); i0 < p.N; i0 += gridDim.y * step) {
+    auto row = [&](int u) { return SHORT ? i0 + u * rows : i0; };
     if constexpr (VEC) {
       float4 f[kIsoUnroll];
 #pragma unroll
       for (int u = 0; u < kIsoUnroll; ++u) {
-        const int64_t x = x0 + (static_cast<int64_t>(u) * kIsoThreads + threadIdx.x) * 4;
-        f[u] = x + 4 <= p.M ? __ldcs(reinterpret_cast<const float4*>(src + x)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        const int64_t x = cell(u), i = row(u);
+        f[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (i < p.N && x + 4 <= p.M) f[u] = __ldcs(reinterpret_cast<const float4*>(p.F + i * p.ld + x));
       }
 #pragma unroll
       for (int u = 0; u < kIsoUnroll; ++u) {
-        const int64_t x = x0 + (static_cast<int64_t>(u) * kIsoThreads + threadIdx.x) * 4;
+        const int64_t x = cell(u), i = row(u);
+        if (i >= p.N) continue;
         if (x + 4 <= p.M) {
-          iso_store4<BF16>(p.U, row + x, iso_map4<KIND>(f[u], p));
+          iso_store4<BF16>(p.U, i * p.ld_out + x, iso_map4<KIND>(f[u], p));
         } else {
           for (int64_t xx = x; xx < p.M; ++xx)
-            iso_store1<BF16>(p.U, row + xx,
-                             iso_value(__ldg(src + xx), p.iso_mode, p.iso_mu, p.iso_inv, p.iso_t));
+            iso_store1<BF16>(p.U, i * p.ld_out + xx,
+                             iso_value(__ldg(p.F + i * p.ld + xx), p.iso_mode, p.iso_mu, p.iso_inv, p.iso_t));
         }
       }
     } else {
       float f[kIsoUnroll];
 #pragma unroll
       for (int u = 0; u < kIsoUnroll; ++u) {
-        const int64_t x = x0 + static_cast<int64_t>(u) * kIsoThreads + threadIdx.x;
-        f[u] = x < p.M ? __ldcs(src + x) : 0.f;
+        const int64_t x = cell(u), i = row(u);
+        f[u] = i < p.N && x < p.M ? __ldcs(p.F + i * p.ld + x) : 0.f;
       }
 #pragma unroll
       for (int u = 0; u < kIsoUnroll; ++u) {
-        const int64_t x = x0 + static_cast<int64_t>(u) * kIsoThreads + threadIdx.x;
-        if (x < p.M)
-          iso_store1<BF16>(p.U, row + x, iso_value(f[u], p.iso_mode, p.iso_mu, p.iso_inv, p.iso_t));
+        const int64_t x = cell(u), i = row(u);
+        if (i < p.N && x < p.M)
+          iso_store1<BF16>(p.U, i * p.ld_out + x, iso_value(f[u], p.iso_mode, p.iso_mu, p.iso_inv, p.iso_t));
       }
     }
   }
+}
+
+template <bool BF16, bool VEC, bool SHORT>
+static void iso_launch_kind(const IsoParams& p, dim3 grid, cudaStream_t s) {
+  if (p.iso_mode == ISO_NORMAL) iso_kernel<BF16, ISO_NORMAL, VEC, SHORT><<<grid, kIsoThreads, 0, s>>>(p);
+  else iso_kernel<BF16, ISO_NONE, VEC, SHORT><<<grid, kIsoThreads, 0, s>>>(p);
 }
 
 template <bool BF16>
@@ -223,14 +236,19 @@ static void iso_launch(const IsoParams& q, cudaStream_t s) {
   const bool vec = (p.N == 1 || ((p.ld & 3) == 0 && (p.ld_out & 3) == 0)) &&
                    (reinterpret_cast<uintptr_t>(p.F) & 15) == 0 &&
                    (reinterpret_cast<uintptr_t>(p.U) & (BF16 ? 7 : 15)) == 0;
-  const int64_t tile = static_cast<int64_t>(kIsoThreads) * kIsoUnroll * (vec ? 4 : 1);
-  const dim3 grid(static_cast<unsigned>((p.M + tile - 1) / tile),
-                  static_cast<unsigned>(p.N < 65535 ? p.N : 65535));
-  const bool normal = p.iso_mode == ISO_NORMAL;
-  if (normal && vec) iso_kernel<BF16, ISO_NORMAL, true><<<grid, kIsoThreads, 0, s>>>(p);
-  else if (normal) iso_kernel<BF16, ISO_NORMAL, false><<<grid, kIsoThreads, 0, s>>>(p);
-  else if (vec) iso_kernel<BF16, ISO_NONE, true><<<grid, kIsoThreads, 0, s>>>(p);
-  else iso_kernel<BF16, ISO_NONE, false><<<grid, kIsoThreads, 0, s>>>(p);
+  // rows of up to one access per thread share a CTA
+  const int64_t accesses = vec ? (p.M + 3) / 4 : p.M;
+  const bool is_short = p.N > 1 && accesses <= kIsoThreads;
+  p.lg_row = 0;
+  while (is_short && (int64_t(1) << p.lg_row) < accesses) ++p.lg_row;
+  const int64_t gx = is_short ? 1 : (accesses + kIsoThreads * kIsoUnroll - 1) / (kIsoThreads * kIsoUnroll);
+  const int64_t per_y = is_short ? int64_t(kIsoThreads >> p.lg_row) * kIsoUnroll : 1;
+  const int64_t gy = (p.N + per_y - 1) / per_y;
+  const dim3 grid(static_cast<unsigned>(gx), static_cast<unsigned>(gy < 65535 ? gy : 65535));
+  if (vec && is_short) iso_launch_kind<BF16, true, true>(p, grid, s);
+  else if (vec) iso_launch_kind<BF16, true, false>(p, grid, s);
+  else if (is_short) iso_launch_kind<BF16, false, true>(p, grid, s);
+  else iso_launch_kind<BF16, false, false>(p, grid, s);
 }
 
 cudaError_t launch_iso(const IsoParams& p, cudaStream_t s) {
