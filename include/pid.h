@@ -202,6 +202,14 @@ pid_status pid_soft_masks_bf16(pid_handle h, const float* F, int64_t N, int64_t 
 pid_status pid_selftest_wait_timeout(pid_handle h, double seconds, void* stream);
 
 /*
+ * pid_selftest_gram_path — diagnostic of the two ways in which the tensor-core Gram of 257 to 512
+ * members is computed, clusters in one pass over the data and row-block tiles over staged operands,
+ * which give the same bits (the paper has no counterpart). `path`: 0 by the library's rule (the
+ * default), 1 tiles, 2 clusters, for the handle's later calls; not for a batch that it already ran.
+ */
+pid_status pid_selftest_gram_path(pid_handle h, int32_t path);
+
+/*
  * pid_contour_bands — the bands of a contour boxplot (Sec. 6) from depths already
  * computed. Every member is binarised, b_i(x) = [u_i(x) > tau], with u_i the soft mask
  * itself (iso == NULL) or the isovalue map of the field (Sec. 3.5). For each cell x, the

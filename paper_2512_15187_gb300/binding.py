@@ -35,7 +35,7 @@ EXPORTS = [
     "pid_serve_stats_get", "pid_serve_stats_reset", "pid_contour_bands", "pid_mean_weighted",
     "pid_spacetime", "pid_depth_from_matrix", "pid_soft_masks_bf16",
     "pid_selftest_wait_timeout", "pid_gram_operands", "pid_serve_cancel",
-    "pid_autotune_shapes", "pid_autotune_describe",
+    "pid_autotune_shapes", "pid_autotune_describe", "pid_selftest_gram_path",
 ]
 PID_KERNEL_STREAM, PID_KERNEL_GRAM, PID_KERNEL_FINALIZE, PID_KERNEL_ISO, PID_KERNEL_BANDS = 0, 1, 2, 3, 4
 PID_KERNEL_GRAM_SPLIT, PID_KERNEL_GRAM_FP8, PID_KERNEL_OPERANDS, PID_KERNEL_SCALE = 5, 6, 7, 8
@@ -122,6 +122,7 @@ def load(path: str = LIB_PATH) -> ctypes.CDLL:
         "pid_soft_masks_bf16": ([P, P, c_int64, c_int64, c_int64, POINTER(pid_iso), P, c_int64, P],
                                 c_int),
         "pid_selftest_wait_timeout": ([P, ctypes.c_double, P], c_int),
+        "pid_selftest_gram_path": ([P, c_int32], c_int),
         "pid_contour_bands": ([P, P, c_int64, c_int64, c_int64, POINTER(pid_iso), P, ctypes.c_double,
                                ctypes.c_double, P, P], c_int),
         "pid_mean": ([P, P, c_int64, c_int64, c_int64, P, P, P, P, P, P], c_int),

@@ -212,7 +212,8 @@ static pid_status to_input(pid_handle h, const pid_ensemble& e, EnsInput* in) {
 // store_u: for exact full PID of a field, pass 1 also writes the soft masks into the
 // workspace and pass 2 streams them (instead of repeating the isovalue map); and the
 // streaming pass of a BF16 tiled-Gram ensemble writes its operands into a buffer of its own
-// (instead of a staging pass into one shared buffer).
+// (instead of a staging pass into one shared buffer), and Gram ensembles for which tiles are the
+// faster take them (instead of clusters, which need no operand planes).
 // steps > 1: the `count` == `steps` records are the time steps of ONE space-time ensemble
 // (4D PID: the cells (x, t) of all steps concatenated). Step t writes its chunk partials
 // right after those of step t - 1, and one finalisation reduces all of them.
@@ -239,7 +240,7 @@ static pid_status plan_batch(pid_handle h, const pid_ensemble* ens, int count, c
     is_lin[e] = in[e].mode == PID_MODE_FULL_LINEAR || (in[e].mode == PID_MODE_FULL && !is_gram[e]);
     tiled[e] = is_gram[e] && in[e].N > kGramMaxN;
     if (tiled[e]) {
-      if ((st = plan_gram_tiled(h, in[e], &tp[e])) != PID_OK) return st;
+      if ((st = plan_gram_tiled(h, in[e], store_u, &tp[e])) != PID_OK) return st;
     } else if (is_gram[e] && (st = plan_gram(h, in[e], &gp[e])) != PID_OK) {
       return st;
     }

@@ -539,6 +539,17 @@ pid_status stream_launch(pid_handle h, StreamParams sp, const StreamCfg& cfg, bo
 // Workspace
 // ---------------------------------------------------------------------------------------
 
+bool workspace_may_hold(pid_handle h, size_t bytes, cudaStream_t s) {
+  if (bytes <= h->ws_bytes) return true;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  cudaStreamIsCapturing(s, &cs);
+  if (cs != cudaStreamCaptureStatusNone) return false;
+  if (h->budget) return bytes + h->fixed_bytes <= h->budget;
+  size_t free_b = 0, total_b = 0;
+  cudaMemGetInfo(&free_b, &total_b);
+  return bytes - h->ws_bytes <= free_b / 2;
+}
+
 pid_status ensure_workspace(pid_handle h, size_t bytes, cudaStream_t s) {
   if (bytes <= h->ws_bytes) return PID_OK;
   if (h->budget && bytes + h->fixed_bytes > h->budget)
@@ -626,13 +637,16 @@ pid_status launch_member_coef_one(pid_handle h, const double* r, int64_t N, floa
 static pid_status run_gram_tiled(pid_handle h, const EnsInput& in, EnsPlan& pl,
                                  const EnsOutputs& out, cudaStream_t s) {
   TiledPlan tp;
-  pid_status st = plan_gram_tiled(h, in, &tp);
+  pid_status st = plan_gram_tiled(h, in, true, &tp);
   if (st != PID_OK) return st;
   const size_t off_sums = pl.part_bytes;
   const size_t off_coef = off_sums + pl.sums_bytes;
   const size_t off_scale = off_coef + pl.coef_bytes;
   const size_t off_gpart = off_scale + kScaleBytes;
   const size_t off_op = off_gpart + tp.gpart_bytes;
+  if (tp.clusters == 0 && !workspace_may_hold(h, off_op + tp.op_bytes, s) &&
+      (st = plan_gram_tiled(h, in, false, &tp)) != PID_OK)
+    return st;
   st = ensure_workspace(h, off_op + tp.op_bytes, s);
   if (st != PID_OK) return st;
   char* ws = static_cast<char*>(h->ws);

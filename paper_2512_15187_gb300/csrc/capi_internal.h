@@ -71,6 +71,7 @@ struct pid_handle_s {
   std::vector<pidh::ProfRecord> prof_captured;   // their events, turned into graph nodes
   bool autotune = false;
   std::map<std::string, std::pair<int, int>> tuned;  // key -> (exchange scheme, ring depth)
+  int gram_path = 0;           // Gram above 256 members: 0 by rule, 1 tiles, 2 clusters (pid_selftest_gram_path)
   std::map<std::string, int> shapes;   // shape key -> tile choice (pid_autotune_shapes)
   std::string tune_file;
 };
@@ -243,7 +244,11 @@ pid_status launch_gram_batch(pid_handle h, const GramPlan& gp, const pidk::EnsDe
                              double bytes, double flops,
                              cudaStream_t s);
 
-pid_status plan_gram_tiled(pid_handle h, const EnsInput& in, TiledPlan* tp);
+// roomy: there is workspace for operand planes where the tiles are the faster.
+pid_status plan_gram_tiled(pid_handle h, const EnsInput& in, bool roomy, TiledPlan* tp);
+// Whether the workspace holds `bytes` or may grow to them: within the budget or, without one, half of
+// the free device memory, and not while the stream is being captured.
+bool workspace_may_hold(pid_handle h, size_t bytes, cudaStream_t s);
 // Operand staging (unless the streaming pass already wrote the BF16 operands) and the
 // tiled Gram launch; `op` holds tp.op_bytes, `gpart` tp.gpart_bytes, `scale`
 // pidk::kScaleBytes (E4M3 member scales).

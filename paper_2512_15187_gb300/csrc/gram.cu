@@ -227,9 +227,32 @@ pid_status launch_gram_batch(pid_handle h, const GramPlan& gp, const EnsDesc* de
 // Row-block-tiled Gram (256 < N <= 512)
 // ---------------------------------------------------------------------------------------
 
+// One pass by clusters once there are chunks for most of them: a chunk keeps one cluster of 3 or 4 SMs
+// busy, a chunk's tiles 2 to 6 SMs (split BF16 512 x 102 400, 25 chunks, 258 us by tiles and 244 by
+// clusters, 400 members 223 and 233; 512 x 5000, 2 chunks, 199 and 264).
 constexpr int kClusterMinChunks = 28;
 
-pid_status plan_gram_tiled(pid_handle h, const EnsInput& in, TiledPlan* tp) {
+// Percent of the 128-row blocks that must be members for the clusters to be the faster. A cluster
+// spends the same time on a block however many members it holds, while the tiles' staging pass takes
+// time by the member; rows off the 16-byte boundary cost the clusters' converters a load per cell; and
+// the tiles of BF16 need no staging pass at all (the streaming pass writes their operands). While
+// every chunk has a cluster of its own, only the loads off the boundary count. Whole calls of 262 144
+// cells, tiles and clusters:
+//   BF16   aligned 257 members 214 and 242 us, 300 227 and 234, 384 267 and 253, 512 432 and 330;
+//          unaligned 300 271 and 306, 390 403 and 452, 512 516 and 454
+//   E4M3   aligned 300 284 and 263, 512 484 and 372; unaligned 257 313 and 352, 390 476 and 499,
+//          512 585 and 513
+//   split  aligned 300 319 and 285; unaligned 257 338 and 364, 300 365 and 361, 512 633 and 524
+// and of 147 456 cells (36 chunks): BF16 aligned 300 178 and 163, unaligned 191 and 207 (257 members).
+static bool clusters_faster(const TiledPlan& tp, int64_t N, bool aligned, int clusters) {
+  int min_fill = 0;
+  if (tp.prec == PID_BF16) min_fill = 87;
+  else if (!aligned) min_fill = tp.prec == PID_FP8 ? 80 : 70;
+  if (100 * N >= int64_t(min_fill) * 128 * tp.R) return true;
+  return tp.n_gchunks <= clusters && (aligned || tp.prec == PID_SPLIT_BF16);
+}
+
+pid_status plan_gram_tiled(pid_handle h, const EnsInput& in, bool roomy, TiledPlan* tp) {
   *tp = TiledPlan{};
   if (in.N > kGramTiledMaxN)
     return fail(h, PID_ERR_UNSUPPORTED,
@@ -253,12 +276,10 @@ pid_status plan_gram_tiled(pid_handle h, const EnsInput& in, TiledPlan* tp) {
   chunk = std::min<int64_t>(std::max<int64_t>(chunk, 4096), 65536);
   tp->chunk_cells = chunk;
   tp->n_gchunks = static_cast<int>((in.M + chunk - 1) / chunk);
-  // One pass by clusters once there are chunks for most of them (kClusterMinChunks): a chunk keeps
-  // one cluster of 3 or 4 SMs busy, a chunk's tiles 2 to 6 SMs. Whole calls, tiles -> clusters: split
-  // BF16 300 x 131 072 (32 chunks) 255 -> 208 us, 512 x 1 048 576 2335 -> 1545; but 448 x 100 003
-  // (25 chunks) 294 -> 297, 512 x 5000 (2 chunks) 199 -> 264, BF16 333 x 100 001 (25 chunks) 197 -> 219.
+  const bool aligned = in.ld % 4 == 0 && reinterpret_cast<uintptr_t>(in.data) % 16 == 0;
   const int clusters = h->gram_clusters[tp->R - 3];
-  if (tp->n_gchunks >= kClusterMinChunks) tp->clusters = std::min(clusters, tp->n_gchunks);
+  const bool by_rule = tp->n_gchunks >= kClusterMinChunks && (!roomy || clusters_faster(*tp, in.N, aligned, clusters));
+  if (h->gram_path == 0 ? by_rule : h->gram_path == 2) tp->clusters = std::min(clusters, tp->n_gchunks);
   const size_t cap = static_cast<size_t>(h->max_smem > 0 ? h->max_smem : 232448);
   tp->stages = 6;
   while (tp->stages > 2 && gram_tiled_smem_bytes(tp->prec, tp->slots, tp->stages) > cap) --tp->stages;

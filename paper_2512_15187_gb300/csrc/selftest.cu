@@ -1,3 +1,4 @@
+// pid_selftest_gram_path: see pid.h.
 // pid_selftest_wait_timeout: exercises the bounded-wait path of the kernels. One thread
 // waits on an mbarrier that nothing arrives at; the bounded wait gives up after the given
 // time and the kernel reports ERR_TIMEOUT in the handle's error word, which the next
@@ -36,5 +37,12 @@ extern "C" pid_status pid_selftest_wait_timeout(pid_handle h, double seconds, vo
       h->err_word, static_cast<uint64_t>(seconds * 1e9));
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(h, e, "wait-timeout kernel launch");
+  return PID_OK;
+}
+
+extern "C" pid_status pid_selftest_gram_path(pid_handle h, int32_t path) {
+  if (!h) return PID_ERR_INVALID_ARG;
+  if (path < 0 || path > 2) return fail(h, PID_ERR_INVALID_ARG, "path must be 0, 1 or 2");
+  h->gram_path = path;
   return PID_OK;
 }
