@@ -417,7 +417,7 @@ static pid_status plan_batch(pid_handle h, const pid_ensemble* ens, int count, c
     }
   }
   bp->work_bytes = off;
-  if (n_logical > kMaxTickets) return fail(h, PID_ERR_UNSUPPORTED, "too many ensembles in one batch");
+  if (n_logical > kMaxBatchItems) return fail(h, PID_ERR_UNSUPPORTED, "too many ensembles in one batch");
   // E4M3 scales of soft masks from a first streaming pass over the same data, where the
   // batch has one: a tiled Gram's own exact-sums pass, or a PID-mean / exact full PID item of
   // the same masks (same pointer, shape, stride and cell measures); otherwise a pass of
@@ -625,7 +625,6 @@ static pid_status enqueue(pid_handle h, const BatchPlan& bp, char* base, const v
       std::memset(&fp, 0, sizeof(fp));
       fp.descs = fdev + L.first;
       fp.n_ens = L.count;
-      fp.err = h->err_word;
       ProfScope ps(h, PID_KERNEL_FINALIZE, 0.0, 0.0, s);
       // the Gram ensembles' launches run beside the others' on a side stream
       BatchCache* c = h->batch;

@@ -402,7 +402,7 @@ pid_status run_blocked(pid_handle h, const EnsInput& in, const EnsOutputs& out, 
   fd.sums = sums;
   fd.block_mass = sums + 3 * N;
   fd.coef = coef;
-  fd.ticket = h->tickets;
+  fd.ticket = h->ticket;
   fd.depth = out.depth ? out.depth : dtmp;
   fd.in_in = out.in_in;
   fd.in_out = out.in_out;

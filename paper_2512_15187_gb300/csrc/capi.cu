@@ -615,7 +615,6 @@ pid_status launch_fin_one(pid_handle h, const FinDesc& fd, cudaStream_t s) {
   fp.one = fd;
   fp.descs = nullptr;
   fp.n_ens = 1;
-  fp.err = h->err_word;
   ProfScope ps(h, PID_KERNEL_FINALIZE, 0.0, 0.0, s);
   cudaError_t e = launch_finalize(fp, l, h->sms, s);
   if (e != cudaSuccess) return cuda_fail(h, e, "finalize launch");
@@ -880,7 +879,8 @@ pid_status pid_create(pid_handle* out, int device, size_t hbm_budget_bytes) {
     delete h;
     return PID_ERR_CUDA;
   }
-  h->fixed_bytes = sizeof(uint32_t) * (1 + kMaxTickets) + 256;
+  for (int R = 3; R <= 4; ++R) h->gram_flag_count = std::max(h->gram_flag_count, h->gram_clusters[R - 3] * R);
+  h->fixed_bytes = 512 + sizeof(unsigned int) * static_cast<size_t>(h->gram_flag_count);
   e = cudaMalloc(&h->fixed, h->fixed_bytes);
   if (e != cudaSuccess) {
     delete h;
@@ -889,7 +889,8 @@ pid_status pid_create(pid_handle* out, int device, size_t hbm_budget_bytes) {
   cudaMemset(h->fixed, 0, h->fixed_bytes);
   h->err_word = static_cast<uint32_t*>(h->fixed);
   load_tune_cache(h);
-  h->tickets = reinterpret_cast<unsigned int*>(static_cast<char*>(h->fixed) + 256);
+  h->ticket = reinterpret_cast<unsigned int*>(static_cast<char*>(h->fixed) + 256);
+  h->gram_flags = reinterpret_cast<unsigned int*>(static_cast<char*>(h->fixed) + 512);
   e = cudaDeviceSynchronize();
   if (e != cudaSuccess) {
     cudaFree(h->fixed);
@@ -926,7 +927,7 @@ pid_status pid_sync(pid_handle h, void* stream) {
   e = cudaMemcpy(&word, h->err_word, sizeof(word), cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return cuda_fail(h, e, "reading the device error word");
   if (word == 0) return PID_OK;
-  cudaMemset(h->fixed, 0, h->fixed_bytes);  // clear the word and any ticket left by an early exit
+  cudaMemset(h->fixed, 0, h->fixed_bytes);  // clear the word and the ticket
   cudaDeviceSynchronize();
   if (word & ERR_TIMEOUT) return fail(h, PID_ERR_TIMEOUT, "a bounded device wait ran out");
   if (word & ERR_DOMAIN) return fail(h, PID_ERR_DOMAIN, "validation: u outside [0,1], NaN, or w <= 0");

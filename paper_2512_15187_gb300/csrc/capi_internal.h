@@ -16,7 +16,7 @@ namespace pidh {
 
 constexpr int64_t kMaxMembers = 512;   // largest N of the fused single-pass kernels
 constexpr int64_t kMaxBlockedMembers = int64_t(1) << 22;   // single calls, member-blocked path
-constexpr int kMaxTickets = 8192;      // ensembles per batch
+constexpr int kMaxBatchItems = 8192;   // ensembles per batch
 constexpr int64_t kMaxMatrixMembers = 65536;   // members of pid_depth_from_matrix
 constexpr int kMaxSpacetimeSteps = 65536;   // time steps of one space-time ensemble
 
@@ -54,10 +54,12 @@ struct pid_handle_s {
   size_t budget = 0;
   void* ws = nullptr;          // growable workspace
   size_t ws_bytes = 0;
-  void* fixed = nullptr;       // error word + tickets (zeroed at creation)
+  void* fixed = nullptr;       // error word, ticket and flags (zeroed at creation)
   size_t fixed_bytes = 0;
   uint32_t* err_word = nullptr;
-  unsigned int* tickets = nullptr;
+  unsigned int* ticket = nullptr;      // of the finalisation above 512 members (zero between calls)
+  unsigned int* gram_flags = nullptr;  // one per CTA of a cluster Gram: accumulators left for the next cluster
+  int gram_flag_count = 0;
   void* desc_dev = nullptr;    // batch descriptor arrays (device)
   void* desc_host = nullptr;   // pinned mirror
   size_t desc_bytes = 0;

@@ -200,8 +200,9 @@ __device__ __forceinline__ void named_barrier(uint32_t id, uint32_t nthreads) {
 
 // ---- dependent launches ----
 // A kernel launched with programmatic stream serialisation may start while the kernel before
-// it still runs: it waits here for that kernel's completion (and its memory) before it
-// touches any global memory. Without the launch attribute this returns at once.
+// it still runs. It waits here for that kernel's completion (and its memory) before it reads what
+// that kernel wrote or writes what it may still read; inputs that neither writes it may load
+// before (the second streaming pass does). Without the launch attribute this returns at once.
 __device__ __forceinline__ void grid_dependency_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }

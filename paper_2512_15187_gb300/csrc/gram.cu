@@ -327,7 +327,9 @@ pid_status launch_gram_tiled_one(pid_handle h, const EnsInput& in, const TiledPl
     cp.vec_ok = in.ld % 4 == 0 && reinterpret_cast<uintptr_t>(in.data) % 16 == 0;
     iso_fill(in.is_field ? &in.iso : nullptr, &cp.iso_mode, &cp.iso_mu, &cp.iso_inv, &cp.iso_t);
     cp.err = h->err_word;
-    cp.flags = h->tickets + kMaxTickets / 2;   // Gram launches of a handle follow one another
+    if (tp.clusters * tp.R > h->gram_flag_count)
+      return fail(h, PID_ERR_UNSUPPORTED, "more clusters than the handle has flags for");
+    cp.flags = h->gram_flags;   // Gram launches of a handle follow one another
     ProfScope ps(h, gram_kind(tp.prec), 4.0 * in.N * in.M + (in.w ? 4.0 * in.M : 0.0), tp.flops, s);
     const cudaError_t e = launch_gram_cluster(cp, in.w, sqrt_w, tp.prec, tp.clusters, s);
     if (e != cudaSuccess) return cuda_fail(h, e, "cluster Gram launch");

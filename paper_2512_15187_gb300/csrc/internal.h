@@ -220,7 +220,6 @@ struct FinParams {
   const FinDesc* descs;
   int32_t n_ens;
   int32_t pad;
-  uint32_t* err;
 };
 
 // What a finalisation launch over several ensembles needs besides the descriptors.

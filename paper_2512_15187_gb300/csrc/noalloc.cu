@@ -136,7 +136,6 @@ extern "C" pid_status pid_mean_noalloc(const float* U, int64_t N, int64_t M, int
   fd.in_out = in_out;
   fd.rank = rank;
   fp.n_ens = 1;
-  fp.err = err_word;
   FinLaunch fl;
   pidh::fin_launch_add(&fl, fd);
   fl.pdl = true;
