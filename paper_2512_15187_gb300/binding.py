@@ -293,9 +293,13 @@ def _ptr(t):
 def _stream(stream):
     if stream is not None:
         return stream.cuda_stream
-    # the current stream's handle without building a torch.cuda.Stream (2.9 us of a small call's 27)
     import torch
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    # the current stream's handle without building a torch.cuda.Stream (2.9 us of a small call's 27),
+    # where torch still has this function of its own
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:
+        return torch.cuda.current_stream().cuda_stream
+    return raw(torch.cuda.current_device())
 
 
 def _check_matrix(x, name):
