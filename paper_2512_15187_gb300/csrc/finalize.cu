@@ -675,7 +675,9 @@ cudaError_t fin_try(const FinParams& p, const FinLaunch& l, int sms, bool pdl, b
 
 // CTAs per ensemble: the most that let every ensemble start at once. An ensemble's chain of barriers
 // and round trips gets shorter with more CTAs, but a second wave of ensembles waits for all of the
-// first one's. More ensembles than that take one CTA each (Gram: the fewest that hold its rows).
+// first one's. More ensembles than that take one CTA each; two or four if some have more than 128 or 256
+// members, for which all the others would wait (200 x (20 x 4096) with 3 x (512 x 20 000) PID-mean, 203
+// ensembles: 145 us with one CTA each, 124 with four), or the fewest that hold the Gram's rows.
 // Batches, eight CTAs each -> this rule: PID-mean of 1000 x (8 x 1024) 198 -> 51 us, of 200 x
 // (20 x 16 384) 149 -> 123; BF16 Gram of 200 x (64 x 4096) 369 -> 123, of 50 x (200 x 8192) 321 -> 264.
 cudaError_t fin_launch_ctas(const FinParams& p, const FinLaunch& l, int sms, bool pdl, cudaStream_t s) {
@@ -686,8 +688,8 @@ cudaError_t fin_launch_ctas(const FinParams& p, const FinLaunch& l, int sms, boo
     if (e == cudaSuccess) e = fin_try<4>(p, l, sms, pdl, false, &done, s);
     if (e == cudaSuccess) e = fin_try<2>(p, l, sms, pdl, false, &done, s);
   }
-  if (e == cudaSuccess) e = fin_try<1>(p, l, sms, pdl, true, &done, s);
-  if (e == cudaSuccess) e = fin_try<2>(p, l, sms, pdl, true, &done, s);
+  if (e == cudaSuccess && (l.gram || l.max_n <= 128)) e = fin_try<1>(p, l, sms, pdl, true, &done, s);
+  if (e == cudaSuccess && (l.gram || l.max_n <= 256)) e = fin_try<2>(p, l, sms, pdl, true, &done, s);
   if (e == cudaSuccess) e = fin_try<4>(p, l, sms, pdl, true, &done, s);
   if (e == cudaSuccess) e = fin_try<8>(p, l, sms, pdl, true, &done, s);
   return e;

@@ -62,7 +62,8 @@ def test_streamed_items(H, mode):
     data = [_dev(_masks(*s)) for s in shapes]
     alone = [H.mean(U) if mode == "mean" else H.full(U, mode="linear") for U in data]
     H.sync()
-    for pick in (list(range(len(shapes))), [0, 1, 2] * 20, list(range(len(shapes))) * 30):
+    for pick in (list(range(len(shapes))), [0, 1, 2] * 20, [0, 2, 3] * 120, ([0, 2, 3] * 3 + [9]) * 40,
+                 list(range(len(shapes))) * 30):
         outs = H.batch([dict(data=data[k], mode=mode) for k in pick])
         H.sync()
         for o, k in zip(outs, pick):
