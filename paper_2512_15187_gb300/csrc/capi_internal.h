@@ -188,7 +188,7 @@ inline void fin_launch_add(pidk::FinLaunch* l, const pidk::FinDesc& fd) {
   l->max_n = fd.N > l->max_n ? fd.N : l->max_n;
   l->gram = l->gram || fd.kind == pidk::FIN_GRAM;
   l->sum_gram = l->sum_gram || (fd.kind == pidk::FIN_GRAM && !fd.gram_inline);
-  l->single = l->single && fd.kind == pidk::FIN_GRAM && pidk::fin_gram_single(fd.N, fd.n_gchunks);
+  l->single = l->single && fd.kind == pidk::FIN_GRAM && pidk::fin_gram_single(fd.N, fd.n_gchunks, fd.n_chunks);
   l->matrix = l->matrix || (fd.P != nullptr && fd.N > pidk::kFinInlineMatrixN);
 }
 pid_status run_blocked(pid_handle h, const EnsInput& in, const EnsOutputs& out, cudaStream_t s);

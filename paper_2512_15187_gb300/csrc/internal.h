@@ -248,11 +248,13 @@ struct IsoParams {
 // 1 TB/s, so 2 MB cost them what the extra launch does.
 inline bool fin_gram_inline(int64_t N, int64_t n_gchunks) { return n_gchunks * N * N * 4 <= (int64_t(2) << 20); }
 // Ensembles that one CTA finalises as fast as a cluster: few members, and chunk sums small enough
-// for one SM. A launch takes one CTA each where that holds for all of its ensembles; the results'
-// bits do not depend on it. One CTA against a cluster of 8: 8 x 4096 16.9 and 22.6 us, 20 x 16 384
-// 18.9 and 22.5, 32 x 4096 20.1 and 22.6, but 64 x 4096 28.4 and 24.1.
-inline bool fin_gram_single(int64_t N, int64_t n_gchunks) {
-  return N <= 32 && n_gchunks * N * N * 4 <= (int64_t(128) << 10);
+// for one SM, both of the Gram and of (m, A), which a streaming pass leaves in many more chunks. A
+// launch takes one CTA each where that holds for all of its ensembles; the results' bits do not depend
+// on it. One CTA against a cluster of 8: 8 x 4096 16.9 and 22.6 us, 20 x 16 384 18.9 and 22.5,
+// 32 x 4096 20.1 and 22.6, but 64 x 4096 28.4 and 24.1; whole E4M3 calls 16 x 65 536 (512 chunks) 52.8
+// and 53.9, but 8 x 300 000 (2344 chunks) 96 and 92.
+inline bool fin_gram_single(int64_t N, int64_t n_gchunks, int64_t n_chunks) {
+  return N <= 32 && n_gchunks * N * N * 4 <= (int64_t(128) << 10) && n_chunks * N <= 8192;
 }
 // Up to this many members the finalisation writes P itself; above, a launch over the whole
 // GPU does (N^2 FP64 products, at 2 per clock and SM).

@@ -98,3 +98,15 @@ def test_many_gram_items(H, count, N, M):
     H.sync()
     for o in outs:
         _same(o, alone, f"{N} x {M}, {count} items")
+
+
+# a Gram item takes a PID-mean or exact item's sums over the same masks: IN_in is bitwise the sibling's
+@pytest.mark.parametrize("prec", ["bf16", "split_bf16", "fp8"])
+@pytest.mark.parametrize("mode", ["mean", "linear"])
+def test_in_in_of_a_sibling(H, prec, mode):
+    for shape in SHAPES:
+        U = _dev(_masks(*shape))
+        a, b = H.batch([dict(data=U, mode=mode), dict(data=U, mode="full", precision=prec)])
+        H.sync()
+        np.testing.assert_array_equal(to_np(a["in_in"]), to_np(b["in_in"]), err_msg=f"{shape} {prec}")
+        np.testing.assert_array_equal(to_np(a["mass"]), to_np(b["mass"]), err_msg=f"{shape} {prec}")
