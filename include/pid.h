@@ -146,7 +146,7 @@ size_t pid_workspace_bytes(pid_handle h);
 typedef enum pid_kernel_kind {
   PID_KERNEL_STREAM = 0,    /* PID-mean / exact full-PID streaming pass */
   PID_KERNEL_GRAM = 1,      /* tensor-core Gram, BF16 operands */
-  PID_KERNEL_FINALIZE = 2,  /* FP64 reduction, depths, ranks */
+  PID_KERNEL_FINALIZE = 2,  /* reduction of the chunk partials, depths, ranks */
   PID_KERNEL_ISO = 3,       /* isovalue map alone */
   PID_KERNEL_BANDS = 4,     /* contour boxplot bands */
   PID_KERNEL_GRAM_SPLIT = 5,  /* tensor-core Gram, split BF16 operands */
@@ -173,8 +173,11 @@ pid_status pid_profile_read(pid_handle h, int kind, pid_kernel_stats* out);
  * events, and keeps the fastest for later launches. That first call synchronises its
  * stream; launches being captured into a CUDA graph are never tuned. If the environment
  * variable PID_AUTOTUNE_CACHE names a file, choices are loaded from it at pid_create and
- * appended to it as they are made. Returns the number of tuned entries in *n_entries
- * (may be NULL).
+ * appended to it as they are made. An entry whose key is not that of a launch is kept and not
+ * used: a key names the kernel class with its stage width (s1 or s2), so entries saved when a class
+ * staged its rows in another width (257 to 384 members: s1 earlier, s2 for aligned rows now) do
+ * not apply, and those launches take the defaults or are tuned again. Returns the number of tuned
+ * entries in *n_entries (may be NULL).
  */
 pid_status pid_autotune_enable(pid_handle h, int enable, int32_t* n_entries);
 
@@ -351,9 +354,10 @@ typedef struct pid_ensemble {
  * the same data, cell measures and isovalue map as an exact-full-PID item of the batch
  * reads that item's first-pass partials instead of streaming the data again; those are
  * bitwise the partials its own pass would write, so this adds no exception.
- * Gram-mode ensembles of 257 to 512 members run the row-block-tiled Gram after their
- * class's streaming launch, one operand-staging and one tile launch each; they share one
- * operand buffer in the workspace, sized for the largest of them.
+ * Gram-mode ensembles of 257 to 512 members run their Gram after their class's streaming
+ * launch: one launch of clusters, or tiles over operands that are staged in one shared
+ * buffer sized for the largest of them or (BF16, where the workspace has room) written by the
+ * streaming launch into a buffer of each ensemble's own. Both ways give the same bits.
  */
 pid_status pid_batch(pid_handle h, const pid_ensemble* ens, int32_t count, void* stream);
 
@@ -456,9 +460,9 @@ pid_status pid_serve_stats_reset(pid_server s);
  * no counterpart; this is an interface convenience.
  *
  * No handle is needed and nothing is allocated: the scratch (per-chunk partial sums, FP64
- * totals, a finalisation ticket and an error word) lives in one fixed 4 MiB array inside
- * the library, which every GPU that loads the library holds until the process exits. The
- * caller still provides U (and w) and the outputs, all device pointers as for pid_mean.
+ * totals and an error word) lives in one fixed 4 MiB array inside the library, which every
+ * GPU that loads the library holds until the process exits. The caller still provides U
+ * (and w) and the outputs, all device pointers as for pid_mean.
  *
  * Limits: N <= 512 and 8 * (4 N + 2 N * n_chunks) + 256 bytes <= 4 MiB, where n_chunks is
  * the number of cell chunks the library splits M into (at most the device's SM count times

@@ -191,8 +191,8 @@ bool encode_1d(CUtensorMap* m, const void* base, uint64_t n, uint32_t box) {
 // Tile class of the streaming kernel as a function of N alone, so that an ensemble is
 // always processed with the same arithmetic order, alone or inside a batch.
 // Each warp holds MPW = ceil(N / G) members x VEC cells in registers (MPW x VEC <= 32);
-// a TMA stage moves sub x T cells of every member (sub = 1 keeps three stages in flight
-// for N up to 512).
+// a TMA stage moves sub x T cells of every member (plan_stream sets sub by the class and how its
+// rows are staged, see stream_sub: the 1 in the table stands for rows that TMA does not load).
 // The streaming tile classes {VEC, G, T, sub, members per warp}, in order of the member rows
 // they hold (G x members per warp). Every member slot of a class costs arithmetic whether
 // or not a member fills it, so the classes above 16 members come in steps that keep the
@@ -631,8 +631,8 @@ pid_status launch_member_coef_one(pid_handle h, const double* r, int64_t N, floa
 
 // Full PID on the tensor cores for 256 < N <= 512: the streaming pass gives the exact
 // PID-mean sums (m_i, N A_i) that calibrate the Gram, the chunk partial Grams come from clusters in
-// one pass over the data or, for short ensembles, from operand rows staged in HBM and the tiled
-// kernel, and the finalisation does the rest.
+// one pass over the data or, where that is the faster (plan_gram_tiled), from operand rows staged in
+// HBM and the tiled kernel, and the finalisation does the rest.
 static pid_status run_gram_tiled(pid_handle h, const EnsInput& in, EnsPlan& pl,
                                  const EnsOutputs& out, cudaStream_t s) {
   TiledPlan tp;

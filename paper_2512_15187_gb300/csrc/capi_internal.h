@@ -141,7 +141,8 @@ struct GramPlan {
 };
 
 // Gram of 256 < N <= 512 members (gram.cu): clusters in one pass over the data (gram_cluster.cu), or,
-// with few chunks, operand rows staged in HBM and a tile of a chunk per CTA (gram_tiled.cu).
+// with few chunks or partly filled row blocks, operand rows staged in HBM and a tile of a chunk per
+// CTA (gram_tiled.cu).
 struct TiledPlan {
   int prec = 0;            // PID_BF16, PID_SPLIT_BF16 or PID_FP8
   int R = 0;               // 128-row blocks

@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(kGramSumThreads) gram_sum_kernel(const __grid_
 // N = 512; rows padded to an odd stride so that the transposed half writes without bank
 // conflicts) and its warps dot them with the scales, which every sweep pushes to all CTAs.
 // Small ensembles with few chunks take one CTA (fin_gram_single): a sweep then costs a CTA barrier
-// instead of a cluster's (20 x 128^2 BF16 with P: 35.0 -> 30.8 us a call).
+// instead of a cluster's (20 x 128^2 BF16 with P: 35.0 -> 30.9 us a call).
 // 512 x 2^20 split BF16 with P: the whole call 2806 -> 2411 us against one CTA that did all of
 // this (437 us); the plume step's three items 1076 -> 996 us (131 us).
 template <int C, int PER_SM>

@@ -14,8 +14,8 @@
 //     per cell chunk); split BF16 issues hi.hi + hi.lo + lo.hi;
 //   * converter warps 0-3 (one per TMEM lane quarter) drain each chunk's accumulator with
 //     tcgen05.ld into an FP32 partial Gram halfway through the next chunk, when its last
-//     products have long landed; the finalisation reduces the partials over chunks in FP64
-//     in a fixed order.
+//     products have long landed; the finalisation reduces the partials over chunks in
+//     compensated FP32 in a fixed order.
 //
 // Every wait is bounded; on a time-out the kernel raises the error word, lets its copies
 // and tensor-core work drain (again bounded) and frees its tensor memory before returning.

@@ -23,8 +23,8 @@
 //     columns per instruction), and four warps drain it into the chunk's partial Gram,
 //     writing both G_ij and its mirror G_ji for the off-diagonal blocks.
 //
-// Ensembles with chunks enough for the GPU's clusters take one pass instead (gram_cluster.cu), with
-// the same chunks and the same bits.
+// Ensembles with chunks enough for the GPU's clusters and well filled row blocks take one pass
+// instead (gram_cluster.cu; the rule is in gram.cu), with the same chunks and the same bits.
 //
 // The exact PID-mean sums (m_i, A_i) that calibrate the Gram come from the streaming
 // kernel's pass over the same ensemble. Every wait is bounded; on a time-out the kernel
