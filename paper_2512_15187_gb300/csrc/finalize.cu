@@ -63,9 +63,15 @@ struct FinShared {
   double csum[kFinBlocks];              // every block's share of the mean contour's mass
   unsigned long long key[kFinMaxN];     // order keys of all depths
 };
-// Partial column sums of a CTA's blocks (dynamic shared memory).
+// Partial column sums of a CTA's blocks (dynamic shared memory): [columns][row groups + 1]. The pad
+// keeps both the lanes that write a row group's columns and those that read a column's groups on
+// banks of their own.
 template <int C>
-constexpr size_t fin_acc_bytes() { return sizeof(Sum3) * kFinThreads * (kFinBlocks / C); }
+constexpr size_t fin_acc_bytes(int N = kFinMaxN) {
+  int cp = 1;
+  while (cp * kFinBlocks < N) cp *= 2;
+  return sizeof(Sum3) * (kFinBlocks / C) * (kFinThreads + 2 * cp);
+}
 
 // The power of two that holds n >= 1: its exponent.
 __device__ __forceinline__ int ceil_log2(int n) { return 32 - __clz(n - 1); }
@@ -102,7 +108,7 @@ __device__ void fin_reduce(FinShared<C>& sh, Sum3* acc, const float* part, int r
   const int ncol = 1 << lg_ncol, columns = V * ncol;
   const int lg_RG = min(ceil_log2((rows + 7) / 8), ceil_log2(kFinThreads) - lg_ncol);
   const int RG = 1 << lg_RG;
-  const int t = threadIdx.x;
+  const int t = threadIdx.x, pitch = RG + 1;
   const int64_t stride = 2 * static_cast<int64_t>(sp.N);
   // the partials of column c, or nullptr for a slot past the CTA's members
   auto column = [&](int c, int* lm, int* half) -> const float* {
@@ -133,7 +139,7 @@ __device__ void fin_reduce(FinShared<C>& sh, Sum3* acc, const float* part, int r
         r += 8 * RG;
       }
     }
-    acc[e] = s;
+    acc[(e & (columns - 1)) * pitch + ((e >> lg_ncol) / V)] = s;
   }
   __syncthreads();
   const int lg_L = min(5, lg_RG), L = 1 << lg_L;        // lanes that share one column
@@ -142,7 +148,7 @@ __device__ void fin_reduce(FinShared<C>& sh, Sum3* acc, const float* part, int r
     const int c = c0 + (t >> lg_L);
     Sum3 s;
     if (c < columns)
-      for (int k = l; k < RG; k += L) sum3_add(s, acc[k * columns + c]);
+      for (int k = l; k < RG; k += L) sum3_add(s, acc[c * pitch + k]);
     for (int o = L / 2; o > 0; o >>= 1) {     // tree: lane 0 ends with the column's sum
       Sum3 other;
       other.x = __shfl_xor_sync(0xffffffffu, s.x, o);
@@ -150,7 +156,7 @@ __device__ void fin_reduce(FinShared<C>& sh, Sum3* acc, const float* part, int r
       other.z = __shfl_xor_sync(0xffffffffu, s.z, o);
       sum3_add(s, other);
     }
-    if (c < columns && l == 0) acc[c] = s;    // in place of the group 0 that this lane alone read
+    if (c < columns && l == 0) acc[c * pitch] = s;   // in place of the group 0 that this lane alone read
   }
   if (L > 1) __syncthreads();
   // to FP64 with a thread per column (few warps: the FP64 pipe takes 16 clocks an instruction)
@@ -158,8 +164,9 @@ __device__ void fin_reduce(FinShared<C>& sh, Sum3* acc, const float* part, int r
     int lm, half;
     const float* src = column(c, &lm, &half);
     if (src == nullptr) continue;
-    double v = sum3_value(acc[c]);
-    if (!(fabsf(acc[c].x) <= kMaxFloat)) {      // infinities, NaN, or beyond the FP32 range: in FP64
+    const Sum3 total = acc[c * pitch];
+    double v = sum3_value(total);
+    if (!(fabsf(total.x) <= kMaxFloat)) {      // infinities, NaN, or beyond the FP32 range: in FP64
       v = 0.0;
       for (int r = 0; r < rows; ++r) v += static_cast<double>(__ldcg(src + r * stride));
     }
@@ -602,7 +609,7 @@ template <int C>
 constexpr size_t fin_gram_smem(int N) {
   const size_t rows = static_cast<size_t>((N + kFinBlocks - 1) / kFinBlocks) * (kFinBlocks / C);
   const size_t bytes = rows * (N | 1) * sizeof(float);
-  return bytes > fin_acc_bytes<C>() ? bytes : fin_acc_bytes<C>();
+  return bytes > fin_acc_bytes<C>(N) ? bytes : fin_acc_bytes<C>(N);
 }
 
 template <int C>
@@ -657,7 +664,7 @@ cudaError_t fin_try(const FinParams& p, const FinLaunch& l, int sms, bool pdl, b
   if (!l.gram) {
     if (!force && ctas > 2 * sms) return cudaSuccess;
     *done = true;
-    return fin_launch(finalize_kernel<C>, grid, kFinThreads, fin_acc_bytes<C>(), pdl, p, s);
+    return fin_launch(finalize_kernel<C>, grid, kFinThreads, fin_acc_bytes<C>(l.max_n), pdl, p, s);
   }
   const size_t smem = fin_gram_smem<C>(l.max_n);
   if (smem > kFinMaxDynamic) return cudaSuccess;

@@ -251,8 +251,8 @@ inline bool fin_gram_inline(int64_t N, int64_t n_gchunks) { return n_gchunks * N
 // for one SM, both of the Gram and of (m, A), which a streaming pass leaves in many more chunks. A
 // launch takes one CTA each where that holds for all of its ensembles; the results' bits do not depend
 // on it. One CTA against a cluster of 8: 8 x 4096 16.9 and 22.6 us, 20 x 16 384 18.9 and 22.5,
-// 32 x 4096 20.1 and 22.6, but 64 x 4096 28.4 and 24.1; whole E4M3 calls 16 x 65 536 (512 chunks) 52.8
-// and 53.9, but 8 x 300 000 (2344 chunks) 96 and 92.
+// 32 x 4096 20.1 and 22.6, but 64 x 4096 28.4 and 24.1; whole E4M3 calls 16 x 65 536 (512 chunks) 51
+// and 54, but 8 x 300 000 (2344 chunks) 96 and 92.
 inline bool fin_gram_single(int64_t N, int64_t n_gchunks, int64_t n_chunks) {
   return N <= 32 && n_gchunks * N * N * 4 <= (int64_t(128) << 10) && n_chunks * N <= 8192;
 }
