@@ -602,6 +602,7 @@ __global__ void __launch_bounds__(256) gram_matrix_kernel(const __grid_constant_
 namespace {
 
 constexpr int kFinMaxDynamic = 200 * 1024;   // besides at most 23 KB of static shared memory
+constexpr int kFinAlone = 112 * 1024;        // so that no second CTA fits it
 constexpr int kFinTwoDynamic = 88 * 1024;    // so that two CTAs fit an SM
 
 // Dynamic shared memory of the Gram's finalisation: its rows, or the column sums before them.
@@ -614,8 +615,7 @@ constexpr size_t fin_gram_smem(int N) {
 
 template <int C>
 cudaError_t fin_init() {
-  cudaError_t e = cudaFuncSetAttribute(finalize_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(fin_acc_bytes<C>()));
+  cudaError_t e = cudaFuncSetAttribute(finalize_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFinAlone);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(finalize_gram_kernel<C, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFinMaxDynamic);
   if constexpr (C < kFinBlocks) {
@@ -664,7 +664,11 @@ cudaError_t fin_try(const FinParams& p, const FinLaunch& l, int sms, bool pdl, b
   if (!l.gram) {
     if (!force && ctas > 2 * sms) return cudaSuccess;
     *done = true;
-    return fin_launch(finalize_kernel<C>, grid, kFinThreads, fin_acc_bytes<C>(l.max_n), pdl, p, s);
+    // Few ensembles: shared memory for one CTA per SM, or the scheduler packs a cluster's CTAs two to
+    // an SM (10 x (300 x 5000) exact full PID 106.5 -> 102 us). Clusters of eight fill three quarters of
+    // the SMs before the rest lie scattered over the GPCs.
+    const size_t acc = 4 * ctas <= 3 * sms ? size_t(kFinAlone) : fin_acc_bytes<C>(l.max_n);
+    return fin_launch(finalize_kernel<C>, grid, kFinThreads, acc, pdl, p, s);
   }
   const size_t smem = fin_gram_smem<C>(l.max_n);
   if (smem > kFinMaxDynamic) return cudaSuccess;
